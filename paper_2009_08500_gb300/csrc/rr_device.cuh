@@ -18,6 +18,19 @@ template <> struct Tr<double> {
     static __device__ __forceinline__ double two_pi() { return 2.0 * CUDART_PI; }
 };
 
+// The approximate quotient and reciprocal root of normal numbers: the forms without the handling of
+// subnormal operands, with the values of __fdividef and rsqrtf where none occur.
+__device__ __forceinline__ float div_normal(float x, float y) {
+    float r;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Angle of the point (x, y), y >= 0, in [0, pi] (atan2 for the upper half
 // plane): folded onto t = min(y, |x|) / max(y, |x|) in [0, 1], where
 // atan(t) = t P(t^2) with P(u) = 1 + c1 u + ... + c8 u^8.  The coefficients
@@ -27,11 +40,14 @@ template <> struct Tr<double> {
 // the minimax polynomial), in FP64, rounded to FP32 -- a CPU test repeats the
 // fit and compares.  Evaluated in FP32 the result is within 1.4 ulp of atan,
 // 4 ulp with the fast quotient.  Then atan = pi/2 - atan(1/t) above the
-// diagonal and pi - angle for x < 0.
-__device__ __forceinline__ float atan2_upper(float y, float x) {
+// diagonal and pi - angle for x < 0.  below: known to be 0 <= y < x, x normal;
+// normal: the larger of y and |x| known to be above 1e-30 (the same values with
+// less folding).
+__device__ __forceinline__ float atan2_upper(float y, float x, const bool below = false, const bool normal = false) {
     const float ax = fabsf(x);
     const float mx = fmaxf(y, ax), mn = fminf(y, ax);
-    const float t = mx > 1e-30f ? __fdividef(mn, mx) : 0.0f;
+    const float t = below ? div_normal(y, x)
+                          : (normal ? div_normal(mn, mx) : (mx > 1e-30f ? __fdividef(mn, mx) : 0.0f));
     const float u = t * t;
     float p = 2.920693019e-03f;
     p = fmaf(p, u, -1.636793092e-02f);
@@ -43,6 +59,7 @@ __device__ __forceinline__ float atan2_upper(float y, float x) {
     p = fmaf(p, u, -3.333315253e-01f);
     p = fmaf(p, u, 1.0f);
     float a = t * p;
+    if (below) return a;
     if (y > ax) a = CUDART_PIO2_F - a;
     if (x < 0.0f) a = CUDART_PI_F - a;
     return a;

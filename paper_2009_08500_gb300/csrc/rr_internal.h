@@ -195,6 +195,8 @@ struct ModelParams {
     double inv_dk;   // 1 / dk (host FP64)
     double exp_c;    // int_0^1 mu / (e^mu - 1) dmu (disk integral of the exponential law's second term)
     double dg;       // 1 / (ng - 1)
+    int32_t nzin;                          // radial grid: annuli inside zcut,
+    float zcutf, inv_dzf, inv_mucutf;      // and 1 / their width, 1 / mu(zcut) (index guesses)
     double k_small;  // small-planet approximation threshold (0 = off)
     double mu_min;   // mu of the outermost bin mean (the small-planet approximation's limb clamp)
     const double* tab;   // tabulated profiles (device): per passband mu nodes then intensities

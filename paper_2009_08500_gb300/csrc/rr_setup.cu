@@ -1,7 +1,9 @@
 // Set-up kernels: LD profile bases and disk integrals, the (k, g) weight table
 // with its projections, the direct model's per-call weight projections, the
 // small-planet rows, and the per-call, per-parameter-vector records.
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "rr_device.cuh"
 
@@ -531,6 +533,268 @@ __global__ void __launch_bounds__(kDirWarps * 32) rr_direct_table_kernel(
             if (grad) Tdk[b * bstride + o] = (dS[q] - th * dtot) / atot;
         }
     }
+}
+
+// The FP32 pass of the affine laws when the tables fit in shared memory.
+// kDirLanes neighbouring lanes share a g node: a step takes kDirLanes
+// consecutive edges of its band, one area per lane, and then lane q adds the
+// step's bins to basis q (and q + kDirLanes) in edge order, the bins' area
+// differences passed by shuffles, so that every sum is formed in the order and
+// rounding of rr_direct_table_kernel, bit for bit, while the products and
+// compensated sums of the bases run in parallel lanes and the areas of a node
+// spread over several.  Eight nodes of nearly equal bands per warp finish
+// together (a thread per node left 30% of the lanes idle), nodes are numbered
+// through the rows, edges and profiles come from shared memory, and the parts of
+// edge_area that no lane of a warp needs (the closed forms outside the lens, the
+// small-angle series or the arctangent form, the compensated factors when
+// c >= 2k) are skipped by warp votes.  Bound by instruction issue (79% of the
+// slots, 31.6 of 32 lanes).  Measured against a thread per node, quadratic law, 200 +
+// 300 annuli, 200 nodes: 1,000 pvs 328 -> 156 us (with dT/dk 339 -> 170), 16 pvs
+// 117 -> 33; 2,048 pvs 552 -> 338 with dT/dk and shared weights; nonlinear law (five
+// bases: two per lane) 4,096 pvs 953 -> 679; CTAs of 128 threads against 256: 343 and
+// 353 (bands differ, smaller CTAs leave fewer warps waiting for their longest).
+constexpr int kDirLanes = 4;
+constexpr int kDirCta = 128;                             // threads per CTA
+constexpr int kDirNodes = kDirCta / kDirLanes;          // nodes per CTA
+constexpr size_t kDirSmem = 48 * 1024;                  // most shared memory of a CTA
+constexpr int kDirMinNz = 48;                           // fewest annuli
+
+// edge_area for a whole warp: the same operations, with votes in place of selects where the warp agrees.
+// FAR: every lane's node has c >= 2k; in the lens then sin kappa_0 <= k / c <= 1/2, so that angle lies below
+// the diagonal and its segment in the range of the series.
+template <bool FAR>
+__device__ __forceinline__ float edge_area_warp(float r, float k, float c, float inv_c, float inv4c2, bool far,
+                                                float& dk, float& dc) {
+    float p1, p2, s2;
+    if (FAR || far) {
+        const float dr = r - c;
+        p1 = k + dr;
+        p2 = k - dr;
+        s2 = (c + r) - k;
+    } else {
+        p1 = sum3_small(r, k, c);
+        p2 = sum3_small(c, k, r);
+        s2 = sum3_small(c, r, k);
+    }
+    const float s1 = r + k + c;
+    const float P = (p1 * p2) * (s1 * s2);
+    const bool lens = P > 1e-30f;
+    const float K = lens ? P * rsqrt_normal(P) : 0.0f;
+    const float r2 = r * r, k2 = k * k, c2 = c * c;
+    const float drk = r - k;
+    const float x0 = fabsf(drk) < fabsf(c - k) ? fmaf(drk, r + k, c2) : fmaf(c - k, c + k, r2);
+    const float x1 = fabsf(drk) < fabsf(c - r) ? fmaf(-drk, r + k, c2) : fmaf(c - r, c + r, k2);
+    const float kap1 = atan2_upper(K, x1, false, FAR);
+    const float q = K * inv4c2;
+    float seg0;
+    if (FAR) {
+        seg0 = __fmul_rn(r2, seg_phi_small(atan2_upper(K, x0, true)));
+    } else {
+        const float kap0 = atan2_upper(K, x0);
+        seg0 = __fmul_rn(r2, seg_phi_small(kap0));
+        if (__any_sync(0xffffffffu, !(kap0 < 0.75f)))
+            if (!(kap0 < 0.75f)) seg0 = fmaf(r2, kap0, -__fmul_rn(q, x0));
+    }
+    float seg1 = fmaf(k2, kap1, -__fmul_rn(q, x1));
+    if (__any_sync(0xffffffffu, kap1 < 0.75f))
+        if (kap1 < 0.75f) seg1 = __fmul_rn(k2, seg_phi_small(kap1));
+    float a = __fadd_rn(seg0, seg1);
+    float ddk = __fmul_rn(__fmul_rn(2.0f, k), kap1), ddc = __fmul_rn(-K, inv_c);
+    // disjoint and nested circles: one of the vanishing factors, and with it P, is not positive
+    if (__any_sync(0xffffffffu, !lens)) {
+        if (s2 <= 0.0f) { a = CUDART_PI_F * r2; ddk = 0.0f; ddc = 0.0f; }
+        if (p2 <= 0.0f) { a = CUDART_PI_F * k2; ddk = 2.0f * CUDART_PI_F * k; ddc = 0.0f; }
+        if (p1 <= 0.0f) { a = 0.0f; ddk = 0.0f; ddc = 0.0f; }
+    }
+    dk = ddk;
+    dc = ddc;
+    return a;
+}
+
+// Last edge <= x (ze[0] = 0 <= x): a guess from the grid's construction (uniform in r to zcut, in mu
+// beyond), corrected against the edges themselves.
+__device__ __forceinline__ int last_edge(const ModelParams& mp, const float* ze, float x) {
+    int j;
+    if (x < mp.zcutf) {
+        j = (int)(x * mp.inv_dzf);
+    } else {
+        const float m = sqrt_approx(fmaxf((1.0f - x) * (1.0f + x), 0.0f));
+        j = mp.nzin + (int)((1.0f - m * mp.inv_mucutf) * (float)(mp.nz - mp.nzin));
+    }
+    j = max(0, min(j, mp.nz));
+    #pragma unroll 1
+    while (j < mp.nz && ze[j + 1] <= x) ++j;
+    #pragma unroll 1
+    while (j > 0 && ze[j] > x) --j;
+    return j;
+}
+
+// MB: bases per lane and walk (1 or 2)
+template <int MB, bool GRAD>
+__global__ void __launch_bounds__(kDirCta, 1024 / kDirCta) rr_direct_lanes_kernel(
+        ModelParams mp, const double* __restrict__ params, const float* __restrict__ zeg,
+        const float* __restrict__ basis, const double* __restrict__ basis64, const float* __restrict__ pre,
+        const float* __restrict__ pre_lo, DirectTables D) {
+    extern __shared__ float dsh[];
+    const int ng = mp.ng, nz = mp.nz, nb_all = mp.nbasis;
+    const int lane = threadIdx.x & 31, sub = lane % kDirLanes;
+    float* ze = dsh;                               // nz + 1 edges
+    float* lb = dsh + ((nz + 4) & ~3);              // profiles, [bin][basis] over groups of kDirLanes bases
+    const int ngrp = (nb_all + kDirLanes - 1) / kDirLanes;
+    for (int j = threadIdx.x; j <= nz; j += blockDim.x) ze[j] = __ldg(zeg + j);
+    for (int b = 0; b < ngrp * kDirLanes; ++b)
+        for (int j = threadIdx.x; j < nz; j += blockDim.x)
+            lb[((size_t)(b / kDirLanes) * nz + j) * kDirLanes + b % kDirLanes] =
+                b < nb_all ? __ldg(basis + (size_t)b * nz + j) : 0.0f;
+    __syncthreads();
+    const int nkp = mp.chromatic ? mp.npb : 1;
+    const int rpp = mp.shared ? 1 : nkp;   // rows per pv
+    const bool own = mp.ld_model == RR_LD_TABULATED && mp.chromatic && !mp.shared;   // a row: its passband's table only
+    float* Thi = reinterpret_cast<float*>(D.hi);
+    float* Tdk = reinterpret_cast<float*>(D.dk);
+    const size_t bstride = (size_t)D.nrows * ng;
+    const int src = lane & ~(kDirLanes - 1);       // the node's first lane
+    const long long first = (long long)blockIdx.x * kDirNodes;
+    const int row0 = (int)(first / ng);
+    const int off = (int)(first - (long long)row0 * ng) + threadIdx.x / kDirLanes;
+    int row = row0 + off / ng;
+    const int ig = off % ng;
+    const bool live = row < D.nrows;
+    if (!__any_sync(0xffffffffu, live)) return;
+    row = live ? row : D.nrows - 1;
+    const int pv = row / rpp, slot = row - pv * rpp;
+    double kd;
+    if (mp.shared) {
+        kd = 0.0;
+        bool ok = true;
+        for (int j = 0; j < nkp; ++j) {
+            const double kj = params[(size_t)pv * mp.nparam + 6 + j];
+            ok = ok && kj > 0.0 && kj < 1.0;
+            kd += kj;
+        }
+        kd = ok ? kd / nkp : -1.0;
+    } else {
+        kd = params[(size_t)pv * mp.nparam + 6 + slot];
+    }
+    const size_t o = (size_t)row * ng + ig;
+    const bool valid = live && kd > 0.0 && kd < 1.0 && !(kd < mp.k_small);
+    const float k = (float)kd;
+    const double gd = ig * mp.dg;
+    const double cd = gd * (1.0 + (double)k);
+    const float c = (float)cd, c_lo = (float)(cd - (double)c), g = (float)gd;
+    const float inv_c = 1.0f / c, inv4c2 = 0.25f * inv_c * inv_c;
+    const bool far = c >= 2.0f * k;
+    float tk = 0.0f, tc = 0.0f;
+    float atot = valid ? edge_area(1.0f, k, c, inv_c, inv4c2, far, tk, tc) : 0.0f;
+    atot += tc * c_lo;
+    const bool walk = valid && ig < ng - 1 && atot > 0.0f;
+    int e0 = 0, nbin = 0;
+    if (walk) {
+        // e0: last edge with ze <= |c - k|; e0 + nbin: first edge after it with ze >= c + k, else nz
+        const float hi_r = c + k;
+        e0 = last_edge(mp, ze, c > k ? c - k : k - c);
+        int e1 = nz;
+        if (hi_r <= 1.0f) {
+            const int j = last_edge(mp, ze, hi_r);
+            e1 = max(e0 + 1, ze[j] >= hi_r ? j : j + 1);
+            while (e1 > e0 + 1 && ze[e1 - 1] >= hi_r) --e1;   // equal edges: the first
+        }
+        nbin = max(min(e1, nz) - e0, 0);
+    }
+    const bool centre = c < k;
+    const float dtot = tk + g * tc;
+    const int steps = __reduce_max_sync(0xffffffffu, (nbin + kDirLanes) / kDirLanes);   // nbin + 1 edges
+    // steps 1 .. full - 1: every bin of the step exists in every node of the warp
+    const int full = __reduce_min_sync(0xffffffffu, (nbin + 1) / kDirLanes);
+    // (c k far from FP32's smallest normals: the FAR form's quotients are of normal numbers)
+    const bool all_far = __all_sync(0xffffffffu, (far && k > 1e-14f) || !walk);
+    for (int b0 = own ? slot : 0; ; b0 += MB * kDirLanes) {
+        const int b_end = own ? slot + 1 : nb_all;
+        // this lane's bases b[m] of the walk and their profile columns
+        int b[MB];
+        const float* lq[MB];
+        DirSum<float> S[MB];
+        float dS[MB];
+        #pragma unroll
+        for (int m = 0; m < MB; ++m) {
+            b[m] = b0 + m * kDirLanes + sub;
+            const int bb = min(b[m], ngrp * kDirLanes - 1);
+            lq[m] = lb + (size_t)(bb / kDirLanes) * nz * kDirLanes + bb % kDirLanes;
+            dS[m] = 0.0f;
+        }
+        float a_last = 0.0f, da_last = 0.0f;   // the last edge of the step before
+        auto steps_loop = [&](auto farc) {
+            #pragma unroll 1
+            for (int s = 0; s < steps; ++s) {
+                const int i = s * kDirLanes + sub;   // edge e0 + i, bin e0 + i - 1
+                float ak, ac;
+                float a = edge_area_warp<decltype(farc)::value>(ze[min(e0 + i, nz)], k, c, inv_c, inv4c2, far, ak, ac);
+                a = fmaf(ac, c_lo, a);
+                const float da = fmaf(g, ac, ak);
+                float ap = __shfl_up_sync(0xffffffffu, a, 1);
+                if (sub == 0) ap = a_last;
+                const float d = a - ap;
+                a_last = __shfl_sync(0xffffffffu, a, src + kDirLanes - 1);
+                float dd = 0.0f;
+                if (GRAD) {
+                    float dap = __shfl_up_sync(0xffffffffu, da, 1);
+                    if (sub == 0) dap = da_last;
+                    dd = da - dap;
+                    da_last = __shfl_sync(0xffffffffu, da, src + kDirLanes - 1);
+                }
+                const int bin0 = s * kDirLanes - 1;
+                const float* lp[MB];
+                #pragma unroll
+                for (int m = 0; m < MB; ++m) lp[m] = lq[m] + (e0 + bin0) * kDirLanes;
+                auto add_bins = [&](auto allc) {
+                    #pragma unroll
+                    for (int t = 0; t < kDirLanes; ++t) {
+                        const float dt = __shfl_sync(0xffffffffu, d, src + t);
+                        const float ddt = GRAD ? __shfl_sync(0xffffffffu, dd, src + t) : 0.0f;
+                        if (decltype(allc)::value || (bin0 + t >= 0 && bin0 + t < nbin)) {
+                            #pragma unroll
+                            for (int m = 0; m < MB; ++m) {
+                                const float v = lp[m][t * kDirLanes];
+                                S[m].add_prod(dt, v);
+                                if (GRAD) dS[m] = fmaf(ddt, v, dS[m]);
+                            }
+                        }
+                    }
+                };
+                if (s > 0 && s < full) add_bins(std::true_type{});
+                else add_bins(std::false_type{});
+            }
+        };
+        if (all_far) steps_loop(std::true_type{});
+        else steps_loop(std::false_type{});
+        #pragma unroll
+        for (int m = 0; m < MB; ++m) {
+            if (live && b[m] < b_end) {
+                const size_t ob = b[m] * bstride + o;
+                if (!walk) {
+                    // g = 1 (no covered area): the row's limit, all weight in the outermost annulus
+                    const double v = valid ? basis64[(size_t)b[m] * nz + nz - 1] : 0.0;
+                    Thi[ob] = (float)v;
+                    D.lo[ob] = (float)(v - (double)(float)v);
+                    if (GRAD) Tdk[ob] = 0.0f;
+                } else {
+                    if (centre) S[m].add(__ldg(pre + (size_t)b[m] * (nz + 1) + e0), __ldg(pre_lo + (size_t)b[m] * (nz + 1) + e0));
+                    float th, tl;
+                    S[m].div(atot, th, tl);
+                    Thi[ob] = th;
+                    D.lo[ob] = tl;
+                    if (GRAD) Tdk[ob] = fmaf(-th, dtot, dS[m]) / atot;
+                }
+            }
+        }
+        if (own || b0 + MB * kDirLanes >= nb_all) break;
+    }
+}
+
+// Shared memory of rr_direct_lanes_kernel.
+static size_t direct_lanes_smem(int nz, int nbasis) {
+    const int ngrp = (nbasis + kDirLanes - 1) / kDirLanes;
+    return ((size_t)((nz + 4) & ~3) + (size_t)ngrp * kDirLanes * nz) * sizeof(float);
 }
 
 // ---------------------------------------------------------------------------
@@ -1288,6 +1552,10 @@ ModelParams model_params(const rr_ctx* c) {
     mp.k_small = c->cfg.k_small;
     mp.mu_min = c->mu.empty() ? 0.0 : c->mu.back();
     mp.nz = c->nz;
+    mp.nzin = c->cfg.nzin;
+    mp.zcutf = (float)c->cfg.zcut;
+    mp.inv_dzf = (float)(c->cfg.nzin / c->cfg.zcut);
+    mp.inv_mucutf = (float)(1.0 / std::sqrt(1.0 - c->cfg.zcut * c->cfg.zcut));
     mp.tab = c->d_tab;
     mp.tab_off = c->d_tab_off;
     // int_0^1 mu / (e^mu - 1) dmu = pi^2/6 - Li2(1/e) + ln(1 - 1/e) (expand 1/(e^mu - 1) = sum_k e^(-k mu));
@@ -1371,6 +1639,18 @@ cudaError_t launch_direct_tables(rr_ctx* c, const double* params, int npv, bool 
         auto kern = p2 ? rr_direct_table_kernel<double, true> : rr_direct_table_kernel<double, false>;
         kern<<<grid, kDirWarps * 32, 0, s>>>(mp, params, c->d_ze, c->d_basis, c->d_basis, c->d_pre64, nullptr,
                                              c->d_lnmu, c->d_mu, D, grad ? 1 : 0);
+    } else if (!p2 && c->nz >= kDirMinNz && direct_lanes_smem(c->nz, c->nbasis) <= kDirSmem) {
+        // the tables fit (up to about 2,400 annuli of four bases: 748 -> 404 us at 2,400 and 500 pvs); on the
+        // coarsest grids, whose bands hold a few edges, a thread per node is the better one (1,000 pvs, 200
+        // nodes: 10 annuli 22 us against 35 here; 75 annuli, 100 nodes 46 against 32 here)
+        const long long nodes = (long long)npv * direct_rows_per_pv(c) * c->cfg.ng;
+        const unsigned blocks = (unsigned)((nodes + kDirNodes - 1) / kDirNodes);
+        const bool own = c->cfg.ld_model == RR_LD_TABULATED && c->cfg.chromatic && !shared_weights(c);
+        const bool one = own || c->nbasis <= kDirLanes;
+        auto kern = grad ? (one ? rr_direct_lanes_kernel<1, true> : rr_direct_lanes_kernel<2, true>)
+                         : (one ? rr_direct_lanes_kernel<1, false> : rr_direct_lanes_kernel<2, false>);
+        kern<<<blocks, kDirCta, direct_lanes_smem(c->nz, c->nbasis), s>>>(
+            mp, params, c->d_zef, c->d_basisf, c->d_basis, c->d_pref, c->d_pref + (size_t)c->nbasis * (c->nz + 1), D);
     } else {
         auto kern = p2 ? rr_direct_table_kernel<float, true> : rr_direct_table_kernel<float, false>;
         kern<<<grid, kDirWarps * 32, 0, s>>>(mp, params, c->d_zef, c->d_basisf, c->d_basis, c->d_pref,
