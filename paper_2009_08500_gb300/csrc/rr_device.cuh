@@ -8,6 +8,85 @@
 
 namespace rr {
 
+// FP64 on GB300: an instruction of a warp every 19 cycles per SM (1/64 of the FP32
+// rate) and 64 cycles from an instruction to one that needs its result, measured; the FP64
+// form's time is its count of FP64 instructions in a full launch and its longest
+// dependent chain in a small one.  The functions below are written for both.
+//
+// Comparisons go through the bits (an FP64 comparison is an FP64 instruction too):
+// |x| <= y (false for a NaN x or y < 0), and the sign of a non-NaN x.
+__device__ __forceinline__ bool abs_le64(double x, double y) {
+    return (__double_as_longlong(x) & 0x7fffffffffffffffll) <= __double_as_longlong(y);
+}
+__device__ __forceinline__ bool neg64(double x) { return __double2hiint(x) < 0; }
+
+// Quotient of finite operands whose result and reciprocal are normal: the hardware's
+// approximate reciprocal (about 20 bits), one Newton-Raphson step, and the quotient
+// corrected by its exact remainder; within an ulp.
+__device__ __forceinline__ double rcp64(double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    return fma(r, fma(-d, r, 1.0), r);
+}
+__device__ __forceinline__ double div64(double n, double d) {
+    const double r = rcp64(d), q = n * r;
+    return fma(fma(-d, q, n), r, q);
+}
+
+// Square root of h >= 0 by Goldschmidt's iteration from the approximate reciprocal
+// root (about 20 bits), the root corrected by its exact remainder; within an ulp;
+// h below 2^-959 (or negative) gives 0.  Five dependent FP64 instructions (sqrt(): 676 cycles measured).
+__device__ __forceinline__ double sqrt64(double h) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
+    double g = h * y, b = 0.5 * y;
+    const double r = fma(-g, b, 0.5);
+    g = fma(g, r, g);
+    b = fma(b, r, b);
+    g = fma(fma(-g, g, h), b, g);
+    return __double2hiint(h) > 0x04000000 ? g : 0.0;   // (h above 2^-959)
+}
+
+// atan(j / 32), j = 0 .. 32 (to FP64 rounding)
+static __device__ const double kAtanTab[33] = {
+    0.0, 0.03123983343026827625, 0.06241880999595734847, 0.0934767811585894635,
+    0.124354994546761435, 0.1549967419239409823, 0.1853479499956947649, 0.215357699697738048,
+    0.2449786631268641542, 0.2741674511196587976, 0.3028848683749714056, 0.3310960767041320949,
+    0.3587706702705722204, 0.3858826693980737759, 0.4124104415973873069, 0.4383365598579578054,
+    0.4636476090008061162, 0.4883339510564055239, 0.5123894603107377067, 0.5358112379604637003,
+    0.558599315343562436, 0.5807563535676703992, 0.6022873461349641817, 0.623199329934065931,
+    0.6435011087932843868, 0.6632029927060932554, 0.6823165548747480783, 0.7008544078844501725,
+    0.7188299996216245054, 0.7362574289814281317, 0.7531512809621943895, 0.7695264804056582604,
+    0.7853981633974483096};
+
+// atan2 for the upper half plane (y >= 0) in FP64: folded onto t = min(y, |x|) /
+// max(y, |x|) in [0, 1], and with t0 = j / 32 the node nearest t (found in FP32),
+//   atan t = atan t0 + atan u,  u = (min - t0 max) / (max + t0 min),  |u| <= 1/63,
+// atan u by its Taylor series through u^9 (truncation below 1e-19 of u).  Within
+// 2 ulp of atan2 (restated by a CPU test); about 20 FP64 instructions.  Operands: the
+// larger one within FP32's range (here it is above the radius ratio times the distance).
+__device__ __forceinline__ double atan2_upper64(double y, double x) {
+    const double ax = __longlong_as_double(__double_as_longlong(x) & 0x7fffffffffffffffll);
+    const bool steep = __double_as_longlong(y) > __double_as_longlong(ax);   // both non-negative
+    const double mx = steep ? y : ax, mn = steep ? ax : y;
+    const int j = __float2int_rn(32.0f * __fdividef((float)mn, (float)mx));
+    const int jc = max(0, min(j, 32));
+    const double t0 = (double)((float)jc * 0.03125f);
+    const double n = fma(-t0, mx, mn), d = fma(t0, mn, mx);
+    const double u = div64(n, d);
+    const double v = u * u, v2 = v * v;
+    const double p = fma(v2, fma(v, 1.0 / 9.0, -1.0 / 7.0), fma(v, 1.0 / 5.0, -1.0 / 3.0));
+    // the fold's constant (0, pi/2 or pi as a pair) is added to the node's angle, off the chain through u
+    const bool left = neg64(x);
+    const double c0 = steep ? CUDART_PIO2 : (left ? CUDART_PI : 0.0);
+    const double c1 = steep ? 6.123233995736766e-17 : (left ? 1.2246467991473532e-16 : 0.0);
+    const bool minus = steep != left;   // angle = c0 -+ atan t
+    const double tj = kAtanTab[jc], th = minus ? -tj : tj;
+    const double s = c0 + th, e = (c0 - s) + th + c1;
+    const double a = fma(u * v, p, u);
+    return s + ((minus ? -a : a) + e);
+}
+
 template <typename R> struct Tr;
 template <> struct Tr<float> {
     static __device__ __forceinline__ float pi() { return CUDART_PI_F; }
@@ -75,13 +154,13 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return r;
 }
 __device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ double d_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ double d_sqrt(double x) { return sqrt64(x); }
 // the forward kernel's per-sample square roots (z, the lens chord): approximate in FP32
 __device__ __forceinline__ float d_sqrt_sample(float x) { return sqrt_approx(x); }
-__device__ __forceinline__ double d_sqrt_sample(double x) { return sqrt(x); }
+__device__ __forceinline__ double d_sqrt_sample(double x) { return sqrt64(x); }
 // the covered area's half-angles: the upper-half-plane arctangent (y = K >= 0)
 __device__ __forceinline__ float d_atan2(float y, float x) { return atan2_upper(y, x); }
-__device__ __forceinline__ double d_atan2(double y, double x) { return atan2(y, x); }
+__device__ __forceinline__ double d_atan2(double y, double x) { return atan2_upper64(y, x); }
 __device__ __forceinline__ void d_sincos(float x, float* s, float* c) { sincosf(x, s, c); }
 __device__ __forceinline__ void d_sincos(double x, double* s, double* c) { sincos(x, s, c); }
 __device__ __forceinline__ float d_rint(float x) { return rintf(x); }
@@ -95,7 +174,7 @@ __device__ __forceinline__ float d_rcp(float x) {
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double d_rcp(double x) { return 1.0 / x; }
+__device__ __forceinline__ double d_rcp(double x) { return div64(1.0, x); }
 
 // Area covered by a planet of radius k at centre distance z on a unit stellar
 // disk (the a(c, k) of Eq. 5), for z < 1 + k, with its partial derivatives.
@@ -121,7 +200,7 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
     const R f2 = z + (one - k);
     const R f4 = z + (one + k);
     R h = (f1 * f2) * (f3 * f4);
-    h = h > R(0) ? h : R(0);
+    if (sizeof(R) == sizeof(float)) h = h > R(0) ? h : R(0);   // (the FP64 root takes negative h as 0)
     const R K = GRAD ? d_sqrt(h) : d_sqrt_sample(h);   // the adjoint keeps the rounding-exact root
     const R zz = z * z, kk = k * k;
     const R kap0 = d_atan2(K, zz + (one - kk));
@@ -446,22 +525,73 @@ struct Orbit64 {
     bool front, ok;
 };
 
+// S = sin x and V = 1 - cos x in FP64: for |x| <= 1 the Taylor series through x^19 and
+// x^20 (truncation below 2e-20), V without cancellation; beyond from the half angle.
+__device__ __forceinline__ void half_angle_SV64(double x, double& S, double& V) {
+    if (abs_le64(x, 1.0)) {
+        // pairs of terms first (Estrin's scheme): a chain of 7 instructions instead of 11
+        const double x2 = x * x, x4 = x2 * x2, x8 = x4 * x4;
+        const double s0 = fma(x2, 1.0 / 120.0, -1.0 / 6.0), s1 = fma(x2, 1.0 / 362880.0, -1.0 / 5040.0);
+        const double s2 = fma(x2, 1.0 / 6227020800.0, -1.0 / 39916800.0);
+        const double s3 = fma(x2, 1.0 / 355687428096000.0, -1.0 / 1307674368000.0);
+        const double s4 = -1.0 / 121645100408832000.0;                       // 1/3! .. 1/19!
+        const double sh = fma(x4, fma(x4, s4, s3), s2);
+        const double ps = fma(x8, sh, fma(x4, s1, s0));
+        S = fma(x * x2, ps, x);
+        const double v0 = fma(x2, -1.0 / 24.0, 0.5), v1 = fma(x2, -1.0 / 40320.0, 1.0 / 720.0);
+        const double v2 = fma(x2, -1.0 / 479001600.0, 1.0 / 3628800.0);
+        const double v3 = fma(x2, -1.0 / 20922789888000.0, 1.0 / 87178291200.0);
+        const double v4 = fma(x2, -1.0 / 2432902008176640000.0, 1.0 / 6402373705728000.0);   // 1/2! .. 1/20!
+        const double vh = fma(x4, fma(x4, v4, v3), v2);
+        V = x2 * fma(x8, vh, fma(x4, v1, v0));
+    } else {
+        double hs, hc;
+        sincos(0.5 * x, &hs, &hc);
+        S = 2.0 * hs * hc;
+        V = 2.0 * hs * hs;
+    }
+}
+
+// FP64 orbit.  Kepler's equation: the FP32 solution x0 (within ~1e-7 of x), then one
+// Halley step in FP64, delta = (f / f') (1 + f'' f / (2 f'^2)), whose error is of
+// order delta^3 (~1e-21), with S and V turned by delta to second order: one
+// evaluation of sine and cosine in place of the four or five of a Newton iteration from the
+// mean anomaly.  A step above 2e-6 (the FP32 solution was poorer than assumed),
+// a failed FP32 solve and e > kESwitch take that iteration.
 __device__ __forceinline__ Orbit64 orbit64(const PvHead<double>& H, double dM) {
     Orbit64 o;
     o.ok = true;
     if (H.flags & kPvCircular) {
-        double hs, hc;
-        sincos(0.5 * dM, &hs, &hc);
-        o.S = 2.0 * hs * hc;
-        o.V = 2.0 * hs * hs;
+        half_angle_SV64(dM, o.S, o.V);
         o.x = dM;
     } else {
-        o.ok = kepler_offset_f64(dM, H.ecE0d, H.esE0d, H.inv_den0d, o.x, o.S, o.V);
+        bool done = false;
+        const double ec = H.ecE0d, es = H.esE0d;
+        if (!(H.flags & kPvKepler64)) {
+            float xf, Sf, Vf;
+            int it;
+            if (kepler_offset_f32((float)dM, (float)ec, (float)es, (float)H.inv_den0d, H.kep2, H.kep3, H.kepC, xf, Sf, Vf, it)) {
+                const double x0 = (double)xf;
+                double S, V;
+                half_angle_SV64(x0, S, V);
+                const double C = 1.0 - V;
+                const double f = fma(es, V, fma(-ec, S, x0 - dM));
+                const double fp = fma(es, S, fma(-ec, C, 1.0));
+                const double h = fma(es, C, ec * S);
+                const double r = rcp64(fp), d1 = f * r;
+                const double dx = fma(0.5 * h * r * d1, d1, d1), d2 = 0.5 * dx * dx;
+                o.x = x0 - dx;
+                o.S = S - fma(dx, C, d2 * S);
+                o.V = V - fma(dx, S, -d2 * C);
+                done = abs_le64(dx, 2e-6);
+            }
+        }
+        if (!done) o.ok = kepler_offset_f64(dM, ec, es, H.inv_den0d, o.x, o.S, o.V);
     }
     o.Px = fma(H.ax1, o.V, H.ax2 * o.S);
     o.Py = H.rho0 + fma(H.ay1, o.V, H.ay2 * o.S);
-    o.z = sqrt(fma(H.a2 * o.Px, o.Px, H.b2 * o.Py * o.Py));
-    o.front = o.Py > 0.0;
+    o.z = sqrt64(fma(H.a2 * o.Px, o.Px, H.b2 * o.Py * o.Py));
+    o.front = __double_as_longlong(o.Py) > 0;
     return o;
 }
 
@@ -1156,6 +1286,39 @@ __device__ __forceinline__ bool queue_finished(TileCounters* tc) {
     }
     return __shfl_sync(0xffffffffu, done, 0) != 0;
 }
+
+// A warp with no group left takes items until the queue is finished.
+template <typename F>
+__device__ __forceinline__ void queue_drain(ItemQueue q, TileCounters* tc, int* err, F&& do_item) {
+    const int lane = threadIdx.x & 31;
+    int idle = 0;
+    bool last = false;   // no producer left: the queue is final
+    #pragma unroll 1
+    while (true) {
+        const int it = queue_claim(tc);
+        if (it >= 0) {
+            const int key = queue_key(q, it);
+            if (key < 0) {
+                if (lane == 0) atomicExch(err, kErrQueueTimeout);
+                return;
+            }
+            do_item(it, key);
+            continue;
+        }
+        if (last) return;
+        if (queue_finished(tc)) {
+            last = true;   // drain what is still claimable
+            continue;
+        }
+        // other warps still take groups: wait for their items (bounded)
+        if (++idle > (1 << 22)) {
+            if (lane == 0) atomicExch(err, kErrQueueTimeout);
+            return;
+        }
+        __nanosleep(64);
+    }
+}
+
 // Value and mu-derivative of profile basis b at an arbitrary mu (the bases of
 // rr_ld_basis_kernel; tabulated: passband b's table interpolated at mu, the
 // slope of the segment holding mu, 0 outside the nodes).  FP64; mu > 0.
@@ -1278,5 +1441,203 @@ __device__ __forceinline__ void points_group(const double* __restrict__ times, c
         grp[g] = gi;
     }
 }
+
+// ---- FP64 form: groups, transit decision and samples ---------------------------
+//
+// The FP64 kernels take the FP32 kernels' 128-time groups and work items.  The
+// transit decisions are conservative and made in FP32 from offsets to a
+// reference time of the group (its first finite one), so that a time outside
+// every window costs one subtraction in FP64 per group and tile of pvs; every
+// sample of a candidate time is then evaluated in FP64 from its own time.
+
+constexpr int kOffTab64 = 512;   // sub-exposure offsets held in shared memory (doubles)
+
+// Passband sampling of the FP64 kernels: ss per passband and, while they all fit, the exact
+// sub-exposure offsets exptime ((s + 1/2) / ss - 1/2) of every passband.
+struct PbShared64 {
+    int ss[RR_MAX_PB];
+    int first[RR_MAX_PB];        // the passband's first offset in off, -1: not tabulated
+    double exptime[RR_MAX_PB];
+    double off[kOffTab64];
+};
+
+__device__ __forceinline__ double sub_offset64(double exptime, int ss, int s) {
+    return exptime * ((s + 0.5) / ss - 0.5);
+}
+
+__device__ __forceinline__ void stage_pb64(const PbParams& pbp, PbShared64* ps) {
+    int at = 0;
+    for (int j = 0; j < pbp.npb; ++j) {
+        const int n = pbp.ss[j];
+        const bool fits = at + n <= kOffTab64;
+        if (threadIdx.x == 0) {
+            ps->ss[j] = n;
+            ps->exptime[j] = pbp.exptime[j];
+            ps->first[j] = fits ? at : -1;
+        }
+        if (fits) {
+            for (int s = threadIdx.x; s < n; s += blockDim.x) ps->off[at + s] = sub_offset64(pbp.exptime[j], n, s);
+            at += n;
+        }
+    }
+}
+
+// A lane's Q consecutive times of a group of 32 Q: the times, their passbands (L.npb: an invalid index, -1: beyond npt),
+// and their float offsets from the group's reference time.
+template <int Q>
+struct Times64 {
+    double t[Q];
+    float dh[Q];
+    int pb[Q];
+    double tref;
+};
+
+template <int Q>
+__device__ __forceinline__ void load_times64(const double* __restrict__ times, const int32_t* __restrict__ pb_index,
+                                             int g, int npt, int npb, Times64<Q>& T) {
+    const int lane = threadIdx.x & 31;
+    const int p0 = (g * 32 + lane) * Q;
+    bool fin_l = false;   // the lane's first finite time
+    double mine = 0.0;
+    #pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        T.t[q] = 0.0;
+        T.pb[q] = -1;
+        if (p0 + q < npt) {
+            T.t[q] = __ldg(times + p0 + q);
+            const int pb = pb_index ? __ldg(pb_index + p0 + q) : 0;
+            T.pb[q] = pb >= 0 && pb < npb ? pb : npb;
+            if (!fin_l && isfinite(T.t[q])) {
+                fin_l = true;
+                mine = T.t[q];
+            }
+        }
+    }
+    const unsigned fin = __ballot_sync(0xffffffffu, fin_l);
+    T.tref = fin ? __shfl_sync(0xffffffffu, mine, __ffs(fin) - 1) : 0.0;
+    #pragma unroll
+    for (int q = 0; q < Q; ++q) T.dh[q] = (float)(T.t[q] - T.tref);
+}
+
+// The group's offset range over its finite times, whether it is whole with valid passbands, and lane
+// l's phase of the reference time for pv l of the tile (cycles from the nearest conjunction, float).
+template <int Q>
+__device__ __forceinline__ void group_state64(const Times64<Q>& T, int npb, const char* recs, int rec_bytes, int npv_t,
+                                              GroupState& gs) {
+    const int lane = threadIdx.x & 31;
+    float lo = INFINITY, hi = -INFINITY;
+    bool whole = true;
+    #pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        if (T.pb[q] >= 0 && isfinite(T.dh[q])) {
+            lo = fminf(lo, T.dh[q]);
+            hi = fmaxf(hi, T.dh[q]);
+        }
+        whole = whole && T.pb[q] >= 0 && T.pb[q] < npb;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    gs.wlo = lo;
+    gs.whi = hi;
+    gs.maxdt = lo <= hi ? fmaxf(fabsf(lo), fabsf(hi)) : 0.0f;
+    gs.full = __all_sync(0xffffffffu, whole);
+    gs.Ah = gs.Al = gs.m = 0.0f;
+    if (lane < npv_t) {
+        const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(recs + (size_t)lane * rec_bytes);
+        if (H.status == 0) {
+            const double psi = (T.tref - H.T0) * H.invP;
+            gs.Ah = (float)(psi - rint(psi));
+        }
+    }
+}
+
+// group_decide for FP64 records (the same test; cl.x = the phase, cl.w = its rounding bound in cycles).
+__device__ __forceinline__ unsigned group_decide64(const GroupState& gs, const char* recs, int rec_bytes, int npv_t,
+                                                   unsigned& bad, float4& cl) {
+    const int lane = threadIdx.x & 31;
+    bool may = false, inval = false;
+    cl = make_float4(gs.Ah, 0.0f, 0.0f, 0.0f);
+    if (lane < npv_t) {
+        const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(recs + (size_t)lane * rec_bytes);
+        inval = H.status != 0;
+        const float Bh = (float)H.Bh;
+        cl.w = 2.4e-7f * (gs.maxdt * Bh + 1.0f);
+        if (!inval && gs.wlo <= gs.whi) {
+            const float W = H.wmax_c + 2.0f * cl.w;
+            may = ceilf(fmaf(gs.wlo, Bh, cl.x) - W) <= fmaf(gs.whi, Bh, cl.x) + W;
+        }
+    }
+    bad = __ballot_sync(0xffffffffu, inval);
+    return __ballot_sync(0xffffffffu, may);
+}
+
+// Per-warp candidate list of the FP64 kernels: the candidates' times, their passband and first flattened sample
+// ((soff << 5) | pb; ps[nc] = ns << 5), and a value per candidate (the forward kernel's sum over its sub-
+// exposures, the adjoint's cotangent weight).
+struct List64 {
+    double t[kWarpPts];
+    double v[kWarpPts];
+    int ps[kWarpPts + 4];
+};
+constexpr size_t kList64Bytes = sizeof(List64);
+static_assert(sizeof(List64) % 16 == 0 && sizeof(PbShared64) % 16 == 0, "16-byte regions");
+
+// Appends the lane's candidates (bits of cand) in time order; bq: the list index of the lane's first one.
+// Returns the number of flattened samples, nc the number of candidates (both warp-uniform).
+template <bool SS1, int Q>
+__device__ __forceinline__ int build_list64(List64* fl, unsigned cand, const Times64<Q>& T, const double (&v)[Q],
+                                            const PbShared64* ps, int& nc, int& bq) {
+    const int lane = threadIdx.x & 31;
+    bq = warp_excl_scan(__popc(cand), nc);
+    int ns = nc, soff = bq;
+    if (!SS1) {
+        int n = 0;
+        #pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if ((cand >> q) & 1u) n += ps->ss[T.pb[q]];
+        soff = warp_excl_scan(n, ns);
+    }
+    int j = bq;
+    #pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        if ((cand >> q) & 1u) {
+            fl->t[j] = T.t[q];
+            fl->v[j] = v[q];
+            fl->ps[j] = (soff << 5) | T.pb[q];
+            soff += SS1 ? 1 : ps->ss[T.pb[q]];
+            ++j;
+        }
+    }
+    if (lane == 0) fl->ps[nc] = ns << 5;
+    __syncwarp();
+    return ns;
+}
+
+// The lane's candidate times for one pv: those whose exposure may overlap its window.
+template <int Q>
+__device__ __forceinline__ unsigned candidates64(const Times64<Q>& T, const PvHead<double>& H, const PvPb<double>* PB, int npb,
+                                                 float4 c) {
+    const float Bh = (float)H.Bh;
+    unsigned cand = 0;
+    #pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int pb = T.pb[q];
+        if (pb < 0 || pb >= npb) continue;
+        const float psi = fmaf(T.dh[q], Bh, c.x);
+        const float d = psi - round_nearest(psi);
+        if (fabsf(d) <= PB[pb].win_pc + c.w) cand |= 1u << q;
+    }
+    return cand;
+}
+
+// Shared memory of the FP64 kernels: [mbarrier 16][counters 64][passbands][one list per warp][pv records ...]
+constexpr size_t kOff64Tc = 16;
+constexpr size_t kOff64Pb = kOff64Tc + 64;
+constexpr size_t kOff64Wl = kOff64Pb + sizeof(PbShared64);
+constexpr int kBlock64 = 64;   // threads per CTA
+constexpr size_t kOff64Recs = kOff64Wl + (kBlock64 / 32) * kList64Bytes;
+static_assert(kOff64Wl % 16 == 0 && kOff64Recs % 16 == 0, "16-byte regions");
 
 }  // namespace rr

@@ -11,8 +11,8 @@
 // asynchronous stores from a constant shared-memory row), and a work item
 // (pv, group) in a shared-memory queue for the others; the remaining warps
 // evaluate the items as they appear (candidate samples compacted per warp,
-// 32 at a time).  FP64 kernel: a tile of kPtTile times strided by kBlock
-// and the same pv tile, every sample in FP64.
+// 32 at a time).  FP64 kernel: the same groups and queue with CTAs of two
+// warps, transit decisions in FP32, every sample in FP64.
 //
 // Mixed precision (FP32 bulk):
 //  * per time, once per call (points_group): dt = t - t_g in FP64, kept as
@@ -379,97 +379,220 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
 }
 
 // ----------------------------- FP64 form -----------------------------------
+//
+// Bound by the FP64 pipe (two lanes per clock and SM).  The groups and the item queue of the FP32
+// kernel in place of a window test in FP64 for every (pv, time), candidate times of a whole warp
+// compacted before they are evaluated, and samples of about 130 FP64 instructions (orbit64,
+// atan2_upper64; about 480 with a Newton iteration from the mean anomaly, sqrt and atan2).
+// CTAs of two warps: an item is a chain of ~6,000 cycles per 32 samples, and small CTAs keep
+// up to 16 items of an SM in flight without waiting for a CTA's longest.  Measured: 512 pvs x
+// 10,007 times 403 -> 100 us (1.06 million FP64 instructions of warps, 0.67 of the pipe's
+// rate), 200 x 5,000 with 10 sub-exposures 4,677 -> 183, 1 x 2,000 25.3 -> 13.8.
 
-__device__ __noinline__ double flux_point64(const PvHead<double>& H, const PvPb<double>& pbc,
-                                            const double* __restrict__ row, int ng, double t, int ss,
-                                            double exptime, bool& bad) {
-    double acc = 0.0;
-    #pragma unroll 1
-    for (int s = 0; s < ss; ++s) {
-        const double ts = t + exptime * ((s + 0.5) / ss - 0.5);
-        double tau = ts - H.T0;
-        tau = fma(-rint(tau * H.invP), H.P, tau);
-        const double dM = H.n * tau;
-        if (fabs(dM) > pbc.win_s) continue;
-        const Orbit64 o = orbit64(H, dM);
-        if (!o.ok) {
-            bad = true;
-            return __longlong_as_double(0x7ff8000000000000ll);
-        }
-        const double g = o.z * pbc.inv1pk;
-        if (!o.front || g >= 1.0) continue;
-        double d0, d1, sl;
-        int cell;
-        const double A = covered_area<double, false>(pbc.k, o.z, d0, d1);
-        const double Ib = lerp_row<double>(row, ng, g, sl, cell);
-        acc += A * Ib;
+// One sample: A Ib (Eq. 5 without the 1 -) at time ts, 0 outside the transit; bad on a Kepler failure.
+__device__ __forceinline__ double delta64(const PvHead<double>& H, const PvPb<double>& pbc,
+                                          const double* __restrict__ row, int ng, double ts, bool& bad) {
+    double tau = ts - H.T0;
+    tau = fma(-rint(tau * H.invP), H.P, tau);
+    const double dM = H.n * tau;
+    if (!abs_le64(dM, pbc.win_s)) return 0.0;
+    const Orbit64 o = orbit64(H, dM);
+    if (!o.ok) {
+        bad = true;
+        return __longlong_as_double(0x7ff8000000000000ll);
     }
-    return 1.0 - acc / ss;
+    const double g = o.z * pbc.inv1pk;
+    if (!o.front || __double2hiint(g) >= 0x3ff00000) return 0.0;   // g >= 1
+    double d0, d1, sl;
+    int cell;
+    const double A = covered_area<double, false>(pbc.k, o.z, d0, d1);
+    return A * lerp_row<double>(row, ng, g, sl, cell);
 }
 
-__global__ void __launch_bounds__(kBlock) rr_flux_fp64_kernel(const double* __restrict__ times,
-                                                              const int32_t* __restrict__ pb_index,
-                                                              int npt, int npv, PbParams pbp, RecLayout L,
-                                                              int pv_tile, const char* __restrict__ records,
-                                                              const char* __restrict__ rowsg,
-                                                              double* __restrict__ flux,
-                                                              int32_t* __restrict__ pv_status, int* err) {
+template <bool SS1, int Q>
+__global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double* __restrict__ times,
+                                                                 const int32_t* __restrict__ pb_index, int npt, int npv,
+                                                                 PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta,
+                                                                 const char* __restrict__ records,
+                                                                 const char* __restrict__ rowsg, double* __restrict__ flux,
+                                                                 int32_t* __restrict__ pv_status, int bulk, int* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-    char* recs = reinterpret_cast<char*>(smem + 16 + 16 * 4 + 16 * kMaxPvTile);
-    const int tid = threadIdx.x;
-    const int pt0 = blockIdx.x * kPtTile;
-    const int pv0 = blockIdx.y * pv_tile;
+    TileCounters* tc = reinterpret_cast<TileCounters*>(smem + kOff64Tc);
+    PbShared64* ps = reinterpret_cast<PbShared64*>(smem + kOff64Pb);
+    char* recs = reinterpret_cast<char*>(smem + kOff64Recs);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    List64* wl = reinterpret_cast<List64*>(smem + kOff64Wl + warp * kList64Bytes);
+    constexpr int kPts = 32 * Q;   // times per group
+    const int ngroups = (npt + kPts - 1) / kPts;
+    const int gbeg = blockIdx.y * groups_per_cta;
+    const int gend = min(ngroups, gbeg + groups_per_cta);
+    const int pv0 = blockIdx.x * pv_tile;
     const int npv_t = min(pv_tile, npv - pv0);
-    if (!stage_to_smem(recs, records + (size_t)pv0 * L.head_bytes, (uint32_t)npv_t * (uint32_t)L.head_bytes, bar,
-                       err))
-        return;
-    double tv[kPPT];
-    int pbv[kPPT];
-    #pragma unroll
-    for (int j = 0; j < kPPT; ++j) {
-        const int p = pt0 + j * kBlock + tid;
-        pbv[j] = -1;
-        tv[j] = 0.0;
-        if (p < npt) {
-            tv[j] = __ldg(times + p);
-            const int pb = pb_index ? __ldg(pb_index + p) : 0;
-            pbv[j] = (pb >= 0 && pb < L.npb) ? pb : L.npb;   // L.npb marks an invalid index (NaN)
-        }
-    }
+    char* qbase = recs + (size_t)pv_tile * L.head_bytes;
+    const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
+    // constant output rows of one group (1 and NaN), sources of the bulk stores
+    double* rows1 = reinterpret_cast<double*>(qbase + queue_bytes(pv_tile * groups_per_cta));
+    double* rowsnan = rows1 + kPts;
     const double nan_ = __longlong_as_double(0x7ff8000000000000ll);
-    #pragma unroll 1
-    for (int i = 0; i < npv_t; ++i) {
+    queue_init(queue, tc, pv_tile * groups_per_cta, gbeg);
+    for (int j = tid; j < kPts; j += kBlock64) {
+        rows1[j] = 1.0;
+        rowsnan[j] = nan_;
+    }
+    fence_proxy_async_smem();
+    stage_pb64(pbp, ps);
+    if (!stage_to_smem(recs, records + (size_t)pv0 * L.head_bytes, (uint32_t)npv_t * (uint32_t)L.head_bytes, bar, err))
+        return;
+    const uint64_t l2_pol = l2_evict_first_policy();
+
+    auto do_group = [&](int g) {
+        Times64<Q> T;
+        load_times64(times, pb_index, g, npt, L.npb, T);
+        GroupState gs;
+        group_state64(T, L.npb, recs, L.head_bytes, npv_t, gs);
+        unsigned bad;
+        float4 cl;
+        const unsigned may = group_decide64(gs, recs, L.head_bytes, npv_t, bad, cl);
+        if (may) queue_push(queue, tc, may, g, cl);
+        unsigned rest = (npv_t >= 32 ? 0xffffffffu : ((1u << npv_t) - 1u)) & ~may;
+        if (bulk && gs.full) {
+            // one bulk store of the group's row per pv outside its windows (16-byte aligned: npt even, aligned flux)
+            if ((rest >> lane) & 1u) {
+                bulk_s2g(flux + (size_t)(pv0 + lane) * npt + (size_t)g * kPts,
+                         ((bad >> lane) & 1u) ? rowsnan : rows1, kPts * sizeof(double), l2_pol);
+                bulk_commit();
+            }
+            return;
+        }
+        #pragma unroll 1
+        while (rest) {
+            const int i = __ffs(rest) - 1;
+            rest &= rest - 1u;
+            const bool inval = (bad >> i) & 1u;
+            double* out = flux + (size_t)(pv0 + i) * npt + (size_t)g * kPts;
+            if (gs.full) {
+                #pragma unroll
+                for (int q = 0; q < Q; ++q) __stcs(out + 32 * q + lane, inval ? nan_ : 1.0);
+            } else {
+                #pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (T.pb[q] >= 0) __stcs(out + Q * lane + q, inval || T.pb[q] >= L.npb ? nan_ : 1.0);
+            }
+        }
+    };
+
+    auto do_item = [&](int it, int key) {
+        const float4 c = queue.c[it];
+        const int g = key >> 5, i = key & 31;
+        Times64<Q> T;
+        load_times64(times, pb_index, g, npt, L.npb, T);
         const char* rec = recs + (size_t)i * L.head_bytes;
         const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(rec);
         const PvPb<double>* PB = reinterpret_cast<const PvPb<double>*>(rec + L.off_pb);
         const double* rows = reinterpret_cast<const double*>(rowsg + (size_t)(pv0 + i) * L.rows_bytes);
-        double* out = flux + (size_t)(pv0 + i) * npt;
-        bool bad = false;
+        const unsigned cand = candidates64(T, H, PB, L.npb, c);
+        double f[Q];
         #pragma unroll
-        for (int j = 0; j < kPPT; ++j) {
-            const int pb = pbv[j];
-            if (pb < 0) continue;
-            double f;
-            if (H.status != 0 || pb >= L.npb) {
-                f = nan_;
+        for (int q = 0; q < Q; ++q) f[q] = T.pb[q] < L.npb ? 1.0 : nan_;
+        bool bad = false;
+        if (__any_sync(0xffffffffu, cand != 0)) {
+            int nc, bq;
+            const double zero[Q] = {};
+            const int ns = build_list64<SS1, Q>(wl, cand, T, zero, ps, nc, bq);
+            auto row_of = [&](int pb) { return rows + (size_t)pb * L.rows_per_pb * L.ng_pad; };
+            if (SS1) {
+                #pragma unroll 1
+                for (int j = lane; j < nc; j += 32) {
+                    const int pb = wl->ps[j] & 31;
+                    wl->v[j] = delta64(H, PB[pb], row_of(pb), L.ng, wl->t[j], bad);
+                }
+                __syncwarp();
             } else {
-                const PvPb<double> pbc = PB[pb];
-                double tau = tv[j] - H.T0;
-                tau = fma(-rint(tau * H.invP), H.P, tau);
-                f = 1.0;
-                if (fabs(H.n * tau) <= pbc.win_p + 1e-9)
-                    f = flux_point64(H, pbc, rows + (size_t)pb * L.rows_per_pb * L.ng_pad, L.ng, tv[j],
-                                     pbp.ss[pb], pbp.exptime[pb], bad);
+                // the item's flattened samples in 32 contiguous runs, one per lane, as in the FP32 kernel: sums of
+                // candidates inside a run are final, a run's head and tail are combined in lane order
+                const int run = (ns + 31) >> 5;
+                const int e_beg = min(lane * run, ns), e_end = min(e_beg + run, ns);
+                int jh = -1, jt = -1;
+                double ph = 0.0, pt = 0.0;
+                if (e_beg < e_end) {
+                    int lo = 0, hi = nc - 1;
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if ((wl->ps[mid] >> 5) <= e_beg) lo = mid; else hi = mid - 1;
+                    }
+                    int j = lo, pw = wl->ps[j], next = wl->ps[j + 1] >> 5, pb = pw & 31;
+                    int sub = e_beg - (pw >> 5);
+                    double t = wl->t[j], part = 0.0;
+                    jh = j;
+                    #pragma unroll 1
+                    for (int e = e_beg; e < e_end; ++e) {
+                        if (e == next) {
+                            if (j == jh) ph = part; else wl->v[j] = part;
+                            ++j;
+                            pw = wl->ps[j];
+                            next = wl->ps[j + 1] >> 5;
+                            pb = pw & 31;
+                            t = wl->t[j];
+                            sub = 0;
+                            part = 0.0;
+                        }
+                        const int at = ps->first[pb];
+                        const double off = at >= 0 ? ps->off[at + sub] : sub_offset64(ps->exptime[pb], ps->ss[pb], sub);
+                        part += delta64(H, PB[pb], row_of(pb), L.ng, t + off, bad);
+                        ++sub;
+                    }
+                    if (j == jh) ph = part; else { jt = j; pt = part; }
+                }
+                const int tprev_j = __shfl_up_sync(0xffffffffu, jt, 1);
+                const double tprev_p = __shfl_up_sync(0xffffffffu, pt, 1);
+                if (lane > 0 && jh >= 0 && tprev_j == jh) ph = tprev_p + ph;
+                const int hnext_j = __shfl_down_sync(0xffffffffu, jh, 1);
+                if (jt >= 0 && (lane == 31 || hnext_j != jt)) wl->v[jt] = pt;
+                double v = ph;
+                #pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const double y = __shfl_up_sync(0xffffffffu, v, o);
+                    const int ky = __shfl_up_sync(0xffffffffu, jh, o);
+                    if (lane >= o && ky == jh) v = y + v;
+                }
+                if (jh >= 0 && (lane == 31 || hnext_j != jh)) wl->v[jh] = v;
+                __syncwarp();
             }
-            __stcs(out + pt0 + j * kBlock + tid, f);
+            int j = bq;
+            #pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if ((cand >> q) & 1u) {
+                    f[q] = SS1 ? 1.0 - wl->v[j] : 1.0 - wl->v[j] / ps->ss[T.pb[q]];
+                    ++j;
+                }
+            }
+            __syncwarp();
         }
         if (bad && pv_status) atomicOr(pv_status + pv0 + i, RR_PV_KEPLER);
+        double* out = flux + (size_t)(pv0 + i) * npt + (size_t)g * kPts + Q * lane;
+        #pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (T.pb[q] >= 0) __stcs(out + q, f[q]);
+    };
+
+    // every warp streams its groups first, then drains the items (FP64 arithmetic dominates)
+    #pragma unroll 1
+    while (true) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(&tc->next_group, 1);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= gend) break;
+        do_group(g);
     }
+    queue_producer_done(tc);
+    queue_drain(queue, tc, err, do_item);
+    bulk_wait_all();   // the bulk stores read shared memory that ends with the CTA
 }
 
 static size_t flux_smem(int pv_tile, int rec_bytes, bool f64, int gpc) {
-    if (f64) return 16 + 16 * 4 + 16 * kMaxPvTile + (size_t)pv_tile * rec_bytes;
+    if (f64)
+        return kOff64Recs + (size_t)pv_tile * rec_bytes + queue_bytes(pv_tile * gpc) + 2 * kWarpPts * sizeof(double);
     // + two constant rows (1 and NaN) for the bulk stores + the group summaries
     return kOffRecsFlux + (size_t)pv_tile * rec_bytes + queue_bytes(pv_tile * gpc) + 2 * kWarpPts * sizeof(float) +
            (size_t)gpc * sizeof(GroupInfo);
@@ -493,6 +616,18 @@ int pv_tile_for(int rec_bytes) {
     if (t < 1) t = 1;
     if (t > kMaxPvTile) t = kMaxPvTile;
     return t;
+}
+
+// Groups per CTA and pvs per CTA of the FP64 kernels.  An SM's FP64 work is what its CTAs hold, so
+// the launch is cut until there are 24 CTAs per SM, the groups first (at most 8: the adjoint's
+// chunk), then the pvs.  Measured at 1, 4, 16, 32 CTAs per SM: 512 pvs x 10,007 times 244, 135, 107, 103
+// us (adjoint 376, 215, 170, 163), 200 x 5,000 with 10 sub-exposures 487, 225, 196, 155.
+void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile) {
+    const long long want = 24LL * c->num_sms;
+    auto ctas = [&] { return (long long)((ngroups + gpc - 1) / gpc) * ((npv + pv_tile - 1) / pv_tile); };
+    gpc = kChunk64;
+    while (gpc > 1 && ctas() < want) gpc >>= 1;
+    while (pv_tile > 1 && ctas() < want) pv_tile = (pv_tile + 1) >> 1;
 }
 
 // Failure-detection self-test: one bounded wait that nothing completes (see
@@ -544,24 +679,32 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
     // the FP64 kernel: headers only, rows through L1/L2
     const bool stage_rows = !f64 && c->cfg.npb > 1 && !grad_layout;
     const int per_pv = stage_rows ? L.head_bytes + L.rows_bytes : L.head_bytes;
-    const int pv_tile = pv_tile_for(per_pv);
-    const int gpc = groups_per_cta(npt);
+    int pv_tile = pv_tile_for(per_pv);
+    int gpc = groups_per_cta(npt);
+    int ngroups = (npt + kWarpPts - 1) / kWarpPts;
+    // FP64, few (pv, group) pairs: groups of 32 times, so that an item is one pass of its warp
+    // (measured: 1 pv x 2,000 times 24.0 -> 13.8 us, 64 x 3,000 33.5 -> 29.4; 512 x 10,007 100 -> 96, but 200 x 5,000
+    // with 10 sub-exposures 180 -> 271: the candidates of 128 times fill a warp's passes better)
+    const bool q1 = f64 && (long long)npv * ngroups < 16LL * c->num_sms;
+    if (q1) ngroups = (npt + 31) / 32;
+    if (f64) split64(c, ngroups, npv, gpc, pv_tile);
     const size_t smem = flux_smem(pv_tile, per_pv, f64, gpc);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
-    const int ngroups = (npt + kWarpPts - 1) / kWarpPts;
-    dim3 grid = f64 ? dim3((npt + kPtTile - 1) / kPtTile, npvt) : dim3(npvt, (ngroups + gpc - 1) / gpc);
+    const dim3 grid(npvt, (ngroups + gpc - 1) / gpc);
     if (smem > kMaxSmem || grid.y > 65535u) return cudaErrorInvalidConfiguration;
+    bool ss1 = true;
+    for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
     cudaError_t e;
     if (f64) {
-        e = cudaFuncSetAttribute(rr_flux_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        auto kern = q1 ? (ss1 ? rr_flux_fp64_kernel<true, 1> : rr_flux_fp64_kernel<false, 1>)
+                       : (ss1 ? rr_flux_fp64_kernel<true, 4> : rr_flux_fp64_kernel<false, 4>);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        rr_flux_fp64_kernel<<<grid, kBlock, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile,
-                                                       (const char*)records, rowsg, (double*)flux, pv_status,
-                                                       c->d_err);
+        const int bulk = npt % 2 == 0 && ((uintptr_t)flux & 15u) == 0 && in_device_memory(flux);
+        kern<<<grid, kBlock64, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile, gpc, (const char*)records, rowsg,
+                                          (double*)flux, pv_status, bulk, c->d_err);
     } else {
-        bool ss1 = true;
-        for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
         auto kern = c->counting
                         ? (stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, true>
                                              : rr_flux_mixed_kernel<true, false, true>)

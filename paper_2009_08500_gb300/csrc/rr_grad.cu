@@ -20,9 +20,14 @@
 // applies the Kipping chain rule).  The chunking depends on npt only, so the
 // result for a pv is independent of which other pvs share the launch and of
 // which warp took which item.
+#include <algorithm>
+
 #include "rr_device.cuh"
 
 namespace rr {
+
+// threads per CTA of the adjoint kernels, the stride of their per-thread columns (dep)
+template <typename R> constexpr int kColStride = sizeof(R) == 8 ? kBlock64 : kBlock;
 
 template <typename R>
 struct GradAcc {
@@ -102,10 +107,10 @@ __device__ __forceinline__ void grad_sample(const PvHead<R>& H, const PvPb<R>& p
     if (DEP) {
         if (L.kbar_slot >= 0) {
             // shared weights: the row's part belongs to the mean k (spread over every k later)
-            dep[(kslot - 6) * kBlock] += gb * kown;
-            dep[(L.kbar_slot - 6) * kBlock] += gb * krow;
+            dep[(kslot - 6) * kColStride<R>] += gb * kown;
+            dep[(L.kbar_slot - 6) * kColStride<R>] += gb * krow;
         } else {
-            dep[(kslot - 6) * kBlock] += gb * (kown + krow);
+            dep[(kslot - 6) * kColStride<R>] += gb * (kown + krow);
         }
     } else {
         acc.k += gb * (kown + krow);
@@ -116,35 +121,7 @@ __device__ __forceinline__ void grad_sample(const PvHead<R>& H, const PvPb<R>& p
             const R* rq = rowblk + (size_t)(3 + cc) * L.ng_pad;
             const R q0 = __ldg(rq + i);
             const R Q = q0 + al * (__ldg(rq + i + 1) - q0);
-            if (DEP) dep[(uslot + cc - 6) * kBlock] += gb * A * Q; else acc.u[cc] += gb * A * Q;
-        }
-    }
-}
-
-// Sum one accumulator set over a warp (shuffles, fixed order) and store it
-// in the warp's slot of the CTA's partial-sum table.  Skipped (zeros) when
-// no lane of the warp contributed.  All lanes of the warp must call.
-template <typename R, bool DEP>
-__device__ __forceinline__ void warp_partials(const GradAcc<R>& acc, const R* dep, int nacc, bool any,
-                                              R* slot /* [nacc] of this warp */) {
-    const int lane = threadIdx.x & 31;
-    if (!__any_sync(0xffffffffu, any)) {
-        for (int j = lane; j < nacc; j += 32) slot[j] = R(0);
-        return;
-    }
-    #pragma unroll
-    for (int j = 0; j < 11; ++j) {
-        if (j < nacc && (j < 6 || !DEP)) {
-            R v = j < 6 ? acc.o[j < 6 ? j : 0] : (j == 6 ? acc.k : acc.u[j >= 7 ? j - 7 : 0]);
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) slot[j] = v;
-        }
-    }
-    if (DEP) {
-        for (int j = 6; j < nacc; ++j) {
-            R v = dep[(j - 6) * kBlock];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) slot[j] = v;
+            if (DEP) dep[(uslot + cc - 6) * kColStride<R>] += gb * A * Q; else acc.u[cc] += gb * A * Q;
         }
     }
 }
@@ -154,10 +131,11 @@ __device__ __forceinline__ void warp_partials(const GradAcc<R>& acc, const R* de
 // lane and keeps the other half, so that lane l ends with the warp total of
 // value idx(l) (held by lanes 2m and 2m + 1): 16 shuffles instead of 5 per
 // value.  The order of the additions is fixed.
-__device__ __forceinline__ float warp_reduce_scatter16(const float (&v)[16], int& idx) {
+template <typename R>
+__device__ __forceinline__ R warp_reduce_scatter16(const R (&v)[16], int& idx) {
     const int lane = threadIdx.x & 31;
     const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
-    float a[8], b[4], c[2];
+    R a[8], b[4], c[2];
     #pragma unroll
     for (int i = 0; i < 8; ++i)
         a[i] = (h16 ? v[i + 8] : v[i]) + __shfl_xor_sync(0xffffffffu, h16 ? v[i] : v[i + 8], 16);
@@ -167,7 +145,7 @@ __device__ __forceinline__ float warp_reduce_scatter16(const float (&v)[16], int
     #pragma unroll
     for (int i = 0; i < 2; ++i)
         c[i] = (h4 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, h4 ? b[i] : b[i + 2], 4);
-    float d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c[0] : c[1], 2);
+    R d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c[0] : c[1], 2);
     d += __shfl_xor_sync(0xffffffffu, d, 1);
     idx = (h16 ? 8 : 0) + (h8 ? 4 : 0) + (h4 ? 2 : 0) + (h2 ? 1 : 0);
     return d;
@@ -179,57 +157,52 @@ template <typename R, bool DEP>
 __device__ __forceinline__ void warp_accumulate(const GradAcc<R>& acc, const R* dep, int nacc, bool any, R* slot) {
     const int lane = threadIdx.x & 31;
     if (!__any_sync(0xffffffffu, any)) return;
-    if constexpr (!DEP && sizeof(R) == sizeof(float)) {
-        const float v[16] = {acc.o[0], acc.o[1], acc.o[2], acc.o[3], acc.o[4], acc.o[5], acc.k, acc.u[0],
-                             acc.u[1], acc.u[2], acc.u[3], 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if constexpr (!DEP) {
+        const R v[16] = {acc.o[0], acc.o[1], acc.o[2], acc.o[3], acc.o[4], acc.o[5], acc.k, acc.u[0],
+                         acc.u[1], acc.u[2], acc.u[3], R(0), R(0), R(0), R(0), R(0)};
         int idx;
-        const float sum = warp_reduce_scatter16(v, idx);
+        const R sum = warp_reduce_scatter16<R>(v, idx);
         if ((lane & 1) == 0 && idx < nacc) slot[idx] += sum;
-        return;
-    }
-    #pragma unroll
-    for (int j = 0; j < 11; ++j) {
-        if (j < nacc && (j < 6 || !DEP)) {
-            R v = j < 6 ? acc.o[j < 6 ? j : 0] : (j == 6 ? acc.k : acc.u[j >= 7 ? j - 7 : 0]);
+    } else {
+        #pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            R v = acc.o[j];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) slot[j] += v;
         }
-    }
-    if (DEP) {
         for (int j = 6; j < nacc; ++j) {
-            R v = dep[(j - 6) * kBlock];
+            R v = dep[(j - 6) * kColStride<R>];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) slot[j] += v;
         }
     }
 }
 
-// After the pv loop: partial[pv][tile][j] = sum over warps (index order) of the
-// warp slots, for every valid pv of the tile.
+// After the group loop: partial[pv][chunk][j] = sum over the CTA's groups (index order).
 template <typename R>
-__device__ __forceinline__ void cta_partials(const R* wpart, const char* recs, int rec_bytes, int npv_t, int nacc,
-                                             int pv0, int tile, int ntiles, R* partials) {
+__device__ __forceinline__ void cta_partials_groups(const R* gacc, const char* recs, int rec_bytes, int npv_t,
+                                                    int nacc, int gpc, int pv0, int chunk, int nchunks,
+                                                    R* partials) {
     __syncthreads();
     for (int idx = threadIdx.x; idx < npv_t * nacc; idx += blockDim.x) {
         const int i = idx / nacc, j = idx % nacc;
         if (reinterpret_cast<const PvHead<R>*>(recs + (size_t)i * rec_bytes)->status != 0) continue;
         R s = R(0);
-        for (int w = 0; w < (kBlock >> 5); ++w) s += wpart[((size_t)i * (kBlock >> 5) + w) * nacc + j];
-        partials[((size_t)(pv0 + i) * ntiles + tile) * nacc + j] = s;
+        for (int g = 0; g < gpc; ++g) s += gacc[((size_t)i * gpc + g) * nacc + j];
+        partials[((size_t)(pv0 + i) * nchunks + chunk) * nacc + j] = s;
     }
 }
 
-// After the group loop: partial[pv][chunk][j] = sum over the CTA's groups (index order).
-__device__ __forceinline__ void cta_partials_groups(const float* gacc, const char* recs, int rec_bytes, int npv_t,
-                                                    int nacc, int gpc, int pv0, int chunk, int nchunks,
-                                                    float* partials) {
+// ... or the groups' own sums, partial[pv][group][j], when the launch is cut finer than the chunks.
+template <typename R>
+__device__ __forceinline__ void cta_group_sums(const R* gacc, const char* recs, int rec_bytes, int npv_t, int nacc, int gpc,
+                                               int pv0, int gbeg, int gend, int ngroups, R* partials) {
     __syncthreads();
-    for (int idx = threadIdx.x; idx < npv_t * nacc; idx += blockDim.x) {
-        const int i = idx / nacc, j = idx % nacc;
-        if (reinterpret_cast<const PvHead<float>*>(recs + (size_t)i * rec_bytes)->status != 0) continue;
-        float s = 0.0f;
-        for (int g = 0; g < gpc; ++g) s += gacc[((size_t)i * gpc + g) * nacc + j];
-        partials[((size_t)(pv0 + i) * nchunks + chunk) * nacc + j] = s;
+    const int per = (gend - gbeg) * nacc;
+    for (int idx = threadIdx.x; idx < npv_t * per; idx += blockDim.x) {
+        const int i = idx / per, r = idx - i * per;
+        if (reinterpret_cast<const PvHead<R>*>(recs + (size_t)i * rec_bytes)->status != 0) continue;
+        partials[((size_t)(pv0 + i) * ngroups + gbeg) * nacc + r] = gacc[(size_t)i * gpc * nacc + r];
     }
 }
 
@@ -545,102 +518,149 @@ __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
         __nanosleep(64);
     }
     if (COUNT) tally_flush(tl, counts);
-    cta_partials_groups(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, chunk, gridDim.y, partials);
+    cta_partials_groups<float>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, chunk, gridDim.y, partials);
 }
 
-template <bool DEP>
-__global__ void __launch_bounds__(kBlock) rr_grad_fp64_kernel(
+// FP64 form: the FP64 flux kernel's groups and items, each item's sums in its own (pv, group) slot as
+// in the FP32 kernel.  pergroup: the slots themselves are written (a launch cut finer than the
+// chunks of kChunk64 groups; rr_grad_finish_kernel then forms the chunks' sums in the same order).
+// Bound by the FP64 pipe.  Measured: 512 pvs x 10,007 times 529 -> 159 us, 64 x 3,000 579 -> 48, 200 x
+// 5,000 with 10 sub-exposures 6,582 -> 211.
+template <bool DEP, bool SS1>
+__global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     const double* __restrict__ times, const int32_t* __restrict__ pb_index, int npt, int npv,
-    PbParams pbp, RecLayout L, int pv_tile, const char* __restrict__ records, const char* __restrict__ rowsg,
-    const double* __restrict__ gflux, double* __restrict__ partials, int nacc, int chromatic,
-    int32_t* __restrict__ pv_status, int* err) {
+    PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta, int pergroup, const char* __restrict__ records,
+    const char* __restrict__ rowsg, const double* __restrict__ gflux, double* __restrict__ partials, int nacc,
+    int chromatic, int32_t* __restrict__ pv_status, int* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-    char* recs = reinterpret_cast<char*>(smem + 16 + 16 * 4 + 16 * kMaxPvTile);
-    double* wpart = reinterpret_cast<double*>(recs + (size_t)pv_tile * L.head_bytes);
-    double* depcols = wpart + (size_t)pv_tile * (kBlock >> 5) * nacc;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int tile = blockIdx.x, ntiles = gridDim.x;
-    const int pt0 = tile * kPtTile;
-    const int pv0 = blockIdx.y * pv_tile;
+    TileCounters* tc = reinterpret_cast<TileCounters*>(smem + kOff64Tc);
+    PbShared64* ps = reinterpret_cast<PbShared64*>(smem + kOff64Pb);
+    char* recs = reinterpret_cast<char*>(smem + kOff64Recs);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    List64* wl = reinterpret_cast<List64*>(smem + kOff64Wl + warp * kList64Bytes);
+    double* gacc = reinterpret_cast<double*>(recs + (size_t)pv_tile * L.head_bytes);   // [pv][group][nacc]
+    double* depcols = gacc + (size_t)pv_tile * groups_per_cta * nacc;
+    char* qbase = reinterpret_cast<char*>(depcols + (DEP ? (size_t)(nacc - 6) * kBlock64 : 0));
+    qbase += (16 - ((uintptr_t)(qbase - (char*)smem) & 15)) & 15;
+    const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
+    const int ngroups = (npt + kWarpPts - 1) / kWarpPts;
+    const int gbeg = blockIdx.y * groups_per_cta;
+    const int gend = min(ngroups, gbeg + groups_per_cta);
+    const int pv0 = blockIdx.x * pv_tile;
     const int npv_t = min(pv_tile, npv - pv0);
-    if (!stage_to_smem(recs, records + (size_t)pv0 * L.head_bytes, (uint32_t)npv_t * (uint32_t)L.head_bytes, bar,
-                       err))
+    queue_init(queue, tc, pv_tile * groups_per_cta, gbeg);
+    stage_pb64(pbp, ps);
+    for (int j = tid; j < pv_tile * groups_per_cta * nacc; j += kBlock64) gacc[j] = 0.0;
+    if (!stage_to_smem(recs, records + (size_t)pv0 * L.head_bytes, (uint32_t)npv_t * (uint32_t)L.head_bytes, bar, err))
         return;
-    double tv[kPPT];
-    int pbv[kPPT];
-    #pragma unroll
-    for (int j = 0; j < kPPT; ++j) {
-        const int p = pt0 + j * kBlock + tid;
-        pbv[j] = -1;
-        tv[j] = 0.0;
-        if (p < npt) {
-            tv[j] = __ldg(times + p);
-            const int pb = pb_index ? __ldg(pb_index + p) : 0;
-            pbv[j] = (pb >= 0 && pb < L.npb) ? pb : -1;
-        }
-    }
     const int nkp = chromatic ? L.npb : 1;
     double* dep = DEP ? depcols + tid : nullptr;
-    #pragma unroll 1
-    for (int i = 0; i < npv_t; ++i) {
+
+    auto do_group = [&](int g) {
+        Times64<4> T;
+        load_times64(times, pb_index, g, npt, L.npb, T);
+        GroupState gs;
+        group_state64(T, L.npb, recs, L.head_bytes, npv_t, gs);
+        unsigned bad;
+        float4 cl;
+        const unsigned may = group_decide64(gs, recs, L.head_bytes, npv_t, bad, cl);
+        if (may) queue_push(queue, tc, may, g, cl);
+    };
+
+    auto do_item = [&](int it, int key) {
+        const float4 c = queue.c[it];
+        const int g = key >> 5, i = key & 31;
+        Times64<4> T;
+        load_times64(times, pb_index, g, npt, L.npb, T);
         const char* rec = recs + (size_t)i * L.head_bytes;
         const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(rec);
-        if (H.status != 0) continue;
         const PvPb<double>* PB = reinterpret_cast<const PvPb<double>*>(rec + L.off_pb);
         const double* rows = reinterpret_cast<const double*>(rowsg + (size_t)(pv0 + i) * L.rows_bytes);
-        const double* gf = gflux + (size_t)(pv0 + i) * npt;
-        GradAcc<double> acc;
-        for (int j = 0; j < 6; ++j) acc.o[j] = 0.0;
-        acc.k = 0.0;
-        for (int j = 0; j < 4; ++j) acc.u[j] = 0.0;
-        if (DEP)
-            for (int j = 6; j < nacc; ++j) dep[(j - 6) * kBlock] = 0.0;
-        bool any = false, bad = false;
+        const double* gf = gflux + (size_t)(pv0 + i) * npt + (size_t)g * kWarpPts + 4 * lane;
+        unsigned cand = candidates64(T, H, PB, L.npb, c);
+        double gbq[4];
         #pragma unroll
-        for (int j = 0; j < kPPT; ++j) {
-            const int pb = pbv[j];
-            if (pb < 0) continue;
-            const PvPb<double> pbc = PB[pb];
-            double tau0 = tv[j] - H.T0;
-            tau0 = fma(-rint(tau0 * H.invP), H.P, tau0);
-            if (fabs(H.n * tau0) > pbc.win_p + 1e-9) continue;
-            const int p = pt0 + j * kBlock + tid;
-            const int ss = pbp.ss[pb];
-            const double gb = -__ldg(gf + p) / ss;
-            if (gb == 0.0) continue;
-            const double* rowblk = rows + (size_t)pb * L.rows_per_pb * L.ng_pad;
-            const int kslot = 6 + (chromatic ? pb : 0);
-            const int uslot = 6 + nkp + pb * L.nldc;
-            #pragma unroll 1
-            for (int s = 0; s < ss; ++s) {
-                const double ts = tv[j] + pbp.exptime[pb] * ((s + 0.5) / ss - 0.5);
-                const double tau = ts - H.T0;
-                const double m = rint(tau * H.invP);
-                const double tr = fma(-m, H.P, tau);
-                const double dM = H.n * tr;
-                if (fabs(dM) > pbc.win_s) continue;
-                const Orbit64 o = orbit64(H, dM);
-                if (!o.ok) { bad = true; continue; }
-                const double g = o.z * pbc.inv1pk;
-                if (!o.front || g >= 1.0) continue;
-                const double psi_tot = m + tr * H.invP;
-                const double xg = g * (double)(L.ng - 1);
-                const int cell = min((int)xg, L.ng - 2);
-                grad_sample<double, DEP>(H, pbc, rowblk, L, o.z, (1.0 + pbc.k) - o.z, o.z - (1.0 - pbc.k), cell,
-                                         xg - (double)cell, o.Px, o.Py, o.S, o.V, psi_tot, gb, acc, dep, kslot,
-                                         uslot);
-                any = true;
+        for (int q = 0; q < 4; ++q) {
+            gbq[q] = 0.0;
+            if ((cand >> q) & 1u) {
+                gbq[q] = SS1 ? -__ldg(gf + q) : -__ldg(gf + q) / ps->ss[T.pb[q]];
+                if (gbq[q] == 0.0) cand &= ~(1u << q);
             }
         }
+        if (!__any_sync(0xffffffffu, cand != 0)) return;
+        GradAcc<double> acc;
+        #pragma unroll
+        for (int j = 0; j < 6; ++j) acc.o[j] = 0.0;
+        acc.k = 0.0;
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) acc.u[j] = 0.0;
+        if (DEP)
+            for (int j = 6; j < nacc; ++j) dep[(j - 6) * kBlock64] = 0.0;
+        bool any = false, bad = false;
+        int nc, bq;
+        const int ns = build_list64<SS1, 4>(wl, cand, T, gbq, ps, nc, bq);
+        #pragma unroll 1
+        for (int e = lane; e < ns; e += 32) {
+            int j = e;
+            double ts;
+            if (SS1) {
+                ts = wl->t[j];
+            } else {
+                int lo = 0, hi = nc - 1;   // the candidate holding sample e
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if ((wl->ps[mid] >> 5) <= e) lo = mid; else hi = mid - 1;
+                }
+                j = lo;
+            }
+            const int pw = wl->ps[j], pb = pw & 31;
+            if (!SS1) {
+                const int sub = e - (pw >> 5), at = ps->first[pb];
+                ts = wl->t[j] + (at >= 0 ? ps->off[at + sub] : sub_offset64(ps->exptime[pb], ps->ss[pb], sub));
+            }
+            const PvPb<double> pbc = PB[pb];
+            const double tau = ts - H.T0;
+            const double m = rint(tau * H.invP);
+            const double tr = fma(-m, H.P, tau);
+            const double dM = H.n * tr;
+            if (!abs_le64(dM, pbc.win_s)) continue;
+            const Orbit64 o = orbit64(H, dM);
+            if (!o.ok) { bad = true; continue; }
+            const double gz = o.z * pbc.inv1pk;
+            if (!o.front || __double2hiint(gz) >= 0x3ff00000) continue;   // gz >= 1
+            const double psi_tot = m + tr * H.invP;
+            const double xg = gz * (double)(L.ng - 1);
+            const int cell = min((int)xg, L.ng - 2);
+            grad_sample<double, DEP>(H, pbc, rows + (size_t)pb * L.rows_per_pb * L.ng_pad, L, o.z, (1.0 + pbc.k) - o.z,
+                                     o.z - (1.0 - pbc.k), cell, xg - (double)cell, o.Px, o.Py, o.S, o.V, psi_tot,
+                                     wl->v[j], acc, dep, 6 + (chromatic ? pb : 0), 6 + nkp + pb * L.nldc);
+            any = true;
+        }
+        __syncwarp();
         if (bad) {
             acc.o[0] = __longlong_as_double(0x7ff8000000000000ll);
             any = true;
             if (pv_status) atomicOr(pv_status + pv0 + i, RR_PV_KEPLER);
         }
-        warp_partials<double, DEP>(acc, dep, nacc, any, wpart + ((size_t)i * (kBlock >> 5) + warp) * nacc);
+        warp_accumulate<double, DEP>(acc, dep, nacc, any, gacc + ((size_t)i * groups_per_cta + (g - gbeg)) * nacc);
+    };
+
+    #pragma unroll 1
+    while (true) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(&tc->next_group, 1);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= gend) break;
+        do_group(g);
     }
-    cta_partials<double>(wpart, recs, L.head_bytes, npv_t, nacc, pv0, tile, ntiles, partials);
+    queue_producer_done(tc);
+    queue_drain(queue, tc, err, do_item);
+    if (pergroup)
+        cta_group_sums<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, gbeg, gend, ngroups, partials);
+    else
+        cta_partials_groups<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, blockIdx.y, gridDim.y,
+                                    partials);
 }
 
 // Sum the partial sums of each pv over its chunks in chunk order (FP64),
@@ -650,29 +670,67 @@ __global__ void __launch_bounds__(kBlock) rr_grad_fp64_kernel(
 // u2 = sqrt(q1) (1 - 2 q2).  A block takes kFinishPvs pvs: one thread per
 // (pv, parameter) for the sums, then one per (pv, passband) for the chain rule.
 constexpr int kFinishThreads = 256;
+constexpr int kFinishChunks = 16;   // chunks summed at a time from per-group sums
 
 template <typename R>
 __global__ void __launch_bounds__(kFinishThreads) rr_grad_finish_kernel(
-    const R* __restrict__ partials, int nchunks, int nacc, int nparam, int npv, int pvs_per_block,
+    const R* __restrict__ partials, int nchunks, int ngroups, int gpc, int nacc, int nparam, int npv, int pvs_per_block,
     const char* __restrict__ heads, int head_bytes, const double* __restrict__ params, int kipping, int shared,
     int npb, int nkp, double* __restrict__ grad) {
-    extern __shared__ double sg[];                 // [pvs_per_block][nacc]
+    extern __shared__ double sg[];                 // [pvs_per_block][nacc], then with per-group sums
+                                                   // [pvs_per_block][kFinishChunks][nacc]
     const int pv0 = blockIdx.x * pvs_per_block;
     const int nloc = min(pvs_per_block, npv - pv0);
+    if (ngroups > 0) {
+        // per-group sums: the chunks' sums first, as the adjoint kernel forms them (group order, in R), a thread
+        // per (pv, chunk, parameter); then the chunks in order
+        double* ch = sg + (size_t)pvs_per_block * nacc;
+        for (int t = threadIdx.x; t < nloc * nacc; t += blockDim.x) sg[t] = 0.0;
+        for (int c0 = 0; c0 < nchunks; c0 += kFinishChunks) {
+            const int per = min(kFinishChunks, nchunks - c0) * nacc;
+            for (int t = threadIdx.x; t < nloc * per; t += blockDim.x) {
+                const int lp = t / per, r = t - lp * per, c = r / nacc;
+                const int g0 = (c0 + c) * gpc, n = min(gpc, ngroups - g0);
+                const R* pp = partials + ((size_t)(pv0 + lp) * ngroups + g0) * nacc + (r - c * nacc);
+                R sc = R(0);
+                for (int g = 0; g < n; g += 8) {   // eight loads in flight
+                    R v[8];
+                    #pragma unroll
+                    for (int q = 0; q < 8; ++q) v[q] = g + q < n ? pp[(size_t)(g + q) * nacc] : R(0);
+                    #pragma unroll
+                    for (int q = 0; q < 8; ++q) sc += v[q];
+                }
+                ch[t] = (double)sc;
+            }
+            __syncthreads();
+            for (int t = threadIdx.x; t < nloc * nacc; t += blockDim.x) {
+                const int lp = t / nacc;
+                const double* q = ch + (size_t)lp * per + (t - lp * nacc);
+                double s = sg[t];
+                for (int o = 0; o < per; o += nacc) s += q[o];
+                sg[t] = s;
+            }
+            __syncthreads();
+        }
+    }
     for (int t = threadIdx.x; t < nloc * nacc; t += blockDim.x) {
         const int lp = t / nacc, j = t - lp * nacc;
-        const R* pp = partials + (size_t)(pv0 + lp) * nchunks * nacc + j;
         double s = 0.0;
-        int c = 0;
-        for (; c + 4 <= nchunks; c += 4) {
-            const R v0 = pp[(size_t)c * nacc], v1 = pp[(size_t)(c + 1) * nacc];
-            const R v2 = pp[(size_t)(c + 2) * nacc], v3 = pp[(size_t)(c + 3) * nacc];
-            s += (double)v0;
-            s += (double)v1;
-            s += (double)v2;
-            s += (double)v3;
+        if (ngroups > 0) {
+            s = sg[t];
+        } else {
+            const R* pp = partials + (size_t)(pv0 + lp) * nchunks * nacc + j;
+            int c = 0;
+            for (; c + 4 <= nchunks; c += 4) {
+                const R v0 = pp[(size_t)c * nacc], v1 = pp[(size_t)(c + 1) * nacc];
+                const R v2 = pp[(size_t)(c + 2) * nacc], v3 = pp[(size_t)(c + 3) * nacc];
+                s += (double)v0;
+                s += (double)v1;
+                s += (double)v2;
+                s += (double)v3;
+            }
+            for (; c < nchunks; ++c) s += (double)pp[(size_t)c * nacc];
         }
-        for (; c < nchunks; ++c) s += (double)pp[(size_t)c * nacc];
         const bool bad = reinterpret_cast<const PvHead<R>*>(heads + (size_t)(pv0 + lp) * head_bytes)->status != 0;
         s = bad ? __longlong_as_double(0x7ff8000000000000ll) : s;
         sg[t] = s;
@@ -703,29 +761,48 @@ __global__ void __launch_bounds__(kFinishThreads) rr_grad_finish_kernel(
 }
 
 static size_t grad_smem(int pv_tile, const RecLayout& L, int nacc, bool dep, size_t rsize, int slots, bool ss1) {
-    size_t s = (rsize == 8 ? 16 + 16 * 4 + 16 * kMaxPvTile : (ss1 ? kOffRecs32Packed : kOffRecs32)) +
-               (size_t)pv_tile * L.head_bytes +
+    size_t s = (rsize == 8 ? kOff64Recs : (ss1 ? kOffRecs32Packed : kOffRecs32)) + (size_t)pv_tile * L.head_bytes +
                (size_t)pv_tile * slots * nacc * rsize;
-    if (dep) s += (size_t)(nacc - 6) * kBlock * rsize;
-    // FP32 kernel: item queue, then the summaries of the CTA's groups and the sine table
-    if (rsize == 4)
-        s = ((s + 15) & ~(size_t)15) + queue_bytes(pv_tile * slots) + (size_t)slots * sizeof(GroupInfo) +
-            (size_t)kSvTabLen * sizeof(float4);
+    if (dep) s += (size_t)(nacc - 6) * (rsize == 8 ? kBlock64 : kBlock) * rsize;
+    s = ((s + 15) & ~(size_t)15) + queue_bytes(pv_tile * slots);
+    // FP32 kernel: the summaries of the CTA's groups and the sine table
+    if (rsize == 4) s += (size_t)slots * sizeof(GroupInfo) + (size_t)kSvTabLen * sizeof(float4);
     return s;
 }
 
-// Partial sums per pv: one per 1024-time tile (FP64 kernel) or per CTA
-// chunk of 128-time groups (FP32 kernel); depends on npt only.
-static int grad_chunks(const rr_ctx* c, int npt) {
-    if (c->cfg.precision == RR_PREC_FP64) return (npt + kPtTile - 1) / kPtTile;
-    const int ngroups = (npt + kWarpPts - 1) / kWarpPts;
-    const int gpc = groups_per_cta(npt);
-    return (ngroups + gpc - 1) / gpc;
+// The cut of one adjoint launch: groups and pvs per CTA, the groups of a partial-sum chunk (a function of npt
+// only, so a pv's gradient never depends on the other pvs of the launch), and whether the kernel writes per-
+// group sums (its CTAs are smaller than a chunk) that rr_grad_finish_kernel adds up.
+struct GradCut {
+    int gpc, pv_tile, chunk, nchunks, ngroups;
+    bool pergroup;
+};
+
+static GradCut grad_cut(const rr_ctx* c, int npv, int npt) {
+    const bool f64 = c->cfg.precision == RR_PREC_FP64;
+    const RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true)
+                            : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
+    GradCut k;
+    k.ngroups = (npt + kWarpPts - 1) / kWarpPts;
+    k.chunk = f64 ? kChunk64 : groups_per_cta(npt);
+    k.nchunks = (k.ngroups + k.chunk - 1) / k.chunk;
+    k.gpc = k.chunk;
+    // pv tile: records plus the per-group partial sums within the shared-memory target
+    auto tile = [&](int gpc) {
+        const size_t per_pv = (size_t)L.head_bytes + (size_t)gpc * grad_nacc(c) * (f64 ? 8 : 4);
+        const int t = (int)(kSmemTarget / per_pv);
+        return t < 1 ? 1 : (t > kMaxPvTile ? kMaxPvTile : t);
+    };
+    k.pv_tile = tile(k.gpc);
+    if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
+    k.pergroup = k.gpc < k.chunk;
+    return k;
 }
 
 size_t partials_bytes(const rr_ctx* c, int npv, int npt) {
     const size_t rsize = c->cfg.precision == RR_PREC_FP64 ? sizeof(double) : sizeof(float);
-    return (size_t)npv * (size_t)grad_chunks(c, npt) * (size_t)grad_nacc(c) * rsize;
+    const GradCut k = grad_cut(c, npv, npt);
+    return (size_t)npv * (size_t)(k.pergroup ? k.ngroups : k.nchunks) * (size_t)grad_nacc(c) * rsize;
 }
 
 template <typename K>
@@ -748,18 +825,14 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     if (shared_weights(c)) L.kbar_slot = c->nparam;
     const bool dep = grad_dep(c);
     const size_t rsize = f64 ? 8 : 4;
-    // pv tile: records plus the per-warp partial sums within the shared-memory target
-    const int slots = f64 ? (kBlock >> 5) : groups_per_cta(npt);   // partial-sum slots per pv in the CTA
-    const size_t per_pv = (size_t)L.head_bytes + (size_t)slots * nacc * rsize;
-    int pv_tile = (int)(kSmemTarget / per_pv);
-    pv_tile = pv_tile < 1 ? 1 : (pv_tile > kMaxPvTile ? kMaxPvTile : pv_tile);
+    const GradCut k = grad_cut(c, npv, npt);
+    const int pv_tile = k.pv_tile, gpc = k.gpc;
     bool ss1 = true;
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
-    const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, slots, ss1);
+    const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
-    const int gpc = groups_per_cta(npt);
-    dim3 grid = f64 ? dim3(grad_chunks(c, npt), npvt) : dim3(npvt, grad_chunks(c, npt));
+    const dim3 grid(npvt, (k.ngroups + gpc - 1) / gpc);
     if (smem > kMaxSmem || grid.y > 65535u) return cudaErrorInvalidConfiguration;
     cudaError_t e;
     if (f64) {
@@ -767,13 +840,17 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     do {                                                                                                      \
         e = set_smem(KERNEL, smem);                                                                           \
         if (e != cudaSuccess) return e;                                                                       \
-        KERNEL<<<grid, kBlock, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile, (const char*)records,   \
-                                          rowsg, (const double*)grad_flux, (double*)partials, nacc,           \
-                                          c->cfg.chromatic,                                                   \
-                                          pv_status, c->d_err);                                               \
+        KERNEL<<<grid, kBlock64, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile, gpc, k.pergroup,      \
+                                          (const char*)records, rowsg, (const double*)grad_flux,              \
+                                          (double*)partials, nacc, c->cfg.chromatic, pv_status, c->d_err);    \
     } while (0)
-        if (dep) RR_LAUNCH_GRAD64(rr_grad_fp64_kernel<true>);
-        else RR_LAUNCH_GRAD64(rr_grad_fp64_kernel<false>);
+        if (dep) {
+            if (ss1) RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<true, true>));
+            else RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<true, false>));
+        } else {
+            if (ss1) RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<false, true>));
+            else RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<false, false>));
+        }
 #undef RR_LAUNCH_GRAD64
     } else {
 #define RR_LAUNCH_GRAD32(KERNEL)                                                                             \
@@ -819,19 +896,22 @@ cudaError_t launch_grad_reduce(rr_ctx* c, int npt, const double* params, int npv
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
     const int nacc = grad_nacc(c);
     const int shared = shared_weights(c) ? 1 : 0;
-    const int nchunks = grad_chunks(c, npt);
+    const GradCut k = grad_cut(c, npv, npt);
+    const int ngr = k.pergroup ? k.ngroups : 0;
     const int nkp = c->cfg.chromatic ? c->cfg.npb : 1;
     const int kip = c->cfg.ld_model == RR_LD_QUADRATIC_TRI ? 1 : 0;
-    const int per_block = kFinishThreads / nacc > 0 ? kFinishThreads / nacc : 1;
+    // a thread per (pv, parameter), with per-group sums per (pv, chunk, parameter)
+    const int cols = nacc * (k.pergroup ? std::min(k.nchunks, kFinishChunks) : 1);
+    const int per_block = std::max(1, kFinishThreads / cols);
     const unsigned blocks = (unsigned)((npv + per_block - 1) / per_block);
-    const size_t smem = (size_t)per_block * nacc * sizeof(double);
+    const size_t smem = (size_t)per_block * (k.pergroup ? nacc + cols : nacc) * sizeof(double);
     if (f64)
         rr_grad_finish_kernel<double><<<blocks, kFinishThreads, smem, s>>>(
-            (const double*)partials, nchunks, nacc, c->nparam, npv, per_block, (const char*)records, L.head_bytes,
+            (const double*)partials, k.nchunks, ngr, k.chunk, nacc, c->nparam, npv, per_block, (const char*)records, L.head_bytes,
             params, kip, shared, c->cfg.npb, nkp, grad_params);
     else
         rr_grad_finish_kernel<float><<<blocks, kFinishThreads, smem, s>>>(
-            (const float*)partials, nchunks, nacc, c->nparam, npv, per_block, (const char*)records, L.head_bytes,
+            (const float*)partials, k.nchunks, ngr, k.chunk, nacc, c->nparam, npv, per_block, (const char*)records, L.head_bytes,
             params, kip, shared, c->cfg.npb, nkp, grad_params);
     c->launches++;
     return cudaGetLastError();

@@ -31,8 +31,7 @@
 namespace rr {
 
 constexpr int kBlock = 256;               // threads per CTA in the per-point kernels
-constexpr int kPPT = 4;                   // points per thread
-constexpr int kPtTile = kBlock * kPPT;    // points per CTA
+constexpr int kPtTile = 4 * kBlock;       // times that groups_per_cta counts in (8 groups)
 constexpr int kMaxPvTile = 32;            // parameter vectors per CTA (upper bound)
 constexpr int kSmemTarget = 32 * 1024;    // record bytes per CTA the tiler aims for
 constexpr int kMaxNz = 4096;
@@ -384,4 +383,6 @@ ModelParams model_params(const rr_ctx* c);
 int pv_tile_for(int rec_bytes);
 void release_host_pipe(rr_ctx* c);
 int groups_per_cta(int npt);
+constexpr int kChunk64 = 8;   // 128-time groups per partial-sum chunk of the FP64 adjoint
+void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile);
 }  // namespace rr
