@@ -77,19 +77,18 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     L.rr_nparam.restype = i32
     L.rr_workspace_bytes.argtypes = [vp, i32, i32, i32]
     L.rr_workspace_bytes.restype = sz
-    L.rr_evaluate.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, sz, vp]
-    L.rr_evaluate_grad.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, vp, sz, vp]
-    L.rr_evaluate_noalloc.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp]
-    L.rr_prepare.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, sz, vp]
-    L.rr_evaluate_prepared.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, sz, vp]
-    L.rr_evaluate_grad_prepared.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, vp, sz,
-                                            vp]
-    L.rr_evaluate_host.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, vp, i32]
-    L.rr_evaluate_both_prepared.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, vp, vp,
-                                            sz, vp]
+    # (the evaluation calls take supersampling and exptime as addresses: see _sampling)
+    L.rr_evaluate.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, sz, vp]
+    L.rr_evaluate_grad.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, sz, vp]
+    L.rr_evaluate_noalloc.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp]
+    L.rr_prepare.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, sz, vp]
+    L.rr_evaluate_prepared.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, sz, vp]
+    L.rr_evaluate_grad_prepared.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, sz, vp]
+    L.rr_evaluate_host.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, i32]
+    L.rr_evaluate_both_prepared.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     L.rr_request_bytes.argtypes = [vp, i32, i32, i32]
     L.rr_request_bytes.restype = sz
-    L.rr_enqueue_host.argtypes = [vp, vp, vp, i32, vp, i32, ctypes.POINTER(i32), dp, vp, vp, vp, vp, vp, sz, vp]
+    L.rr_enqueue_host.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     L.rr_server_create.argtypes = [i32, i32, sz, ctypes.POINTER(vp)]
     L.rr_server_create.restype = ctypes.c_int
     L.rr_server_destroy.argtypes = [vp]
@@ -144,15 +143,22 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle without a Stream object
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     return stream.cuda_stream or None
 
 
 def _host_array(x, n, dtype, default):
+    if type(x) is np.ndarray and x.dtype == dtype and x.shape == (n,) and x.flags.c_contiguous:
+        return x
     if x is None:
         x = [default] * n
-    a = np.ascontiguousarray(np.broadcast_to(np.asarray(x, dtype=dtype), (n,)))
-    return a
+    return np.ascontiguousarray(np.broadcast_to(np.asarray(x, dtype=dtype), (n,)))
+
+
+_I32, _F64 = np.dtype(np.int32), np.dtype(np.float64)
 
 
 class Model:
@@ -195,6 +201,7 @@ class Model:
         if st != 0:
             raise RRError(st, self.lib.rr_last_error(None).decode())
         self._h = h
+        self._nparam = int(self.lib.rr_nparam(h))
         self.dtype = torch.float64 if precision == "fp64" else torch.float32
 
     # -- plumbing -------------------------------------------------------------
@@ -215,7 +222,14 @@ class Model:
 
     @property
     def nparam(self) -> int:
-        return int(self.lib.rr_nparam(self._h))
+        return self._nparam
+
+    def _sampling(self, supersampling, exptime):
+        """Host arrays of the sub-exposure counts and exposure lengths, and their addresses (the arrays are to be
+        kept until the library call, which copies them, has returned)."""
+        ss = _host_array(supersampling, self.npb, _I32, 1)
+        ex = _host_array(exptime, self.npb, _F64, 0.0)
+        return ss, ex, ss.ctypes.data, ex.ctypes.data
 
     @property
     def launch_count(self) -> int:
@@ -301,17 +315,28 @@ class Model:
         self._check(self.lib.rr_selftest_wait(self._h, int(which), _stream_handle(stream)))
 
     # -- evaluation -----------------------------------------------------------
+    # A small call's time is the host's: the argument conversions below are few on purpose (Grace host, one
+    # light curve: 46.7 -> 23.5 us a call, of which the library's two launches take 8).
     def _inputs(self, times, params, pb_index):
         dev = self.device
-        for name, t, dt in (("times", times, torch.float64), ("params", params, torch.float64)):
-            if not (isinstance(t, torch.Tensor) and t.device == dev and t.dtype == dt and t.is_contiguous()):
-                raise TypeError(f"{name} must be a contiguous {dt} tensor on {dev}")
-        if params.dim() != 2 or params.shape[1] != self.nparam:
-            raise ValueError(f"params must have shape (npv, {self.nparam})")
-        if pb_index is not None and not (pb_index.device == dev and pb_index.dtype == torch.int32
-                                         and pb_index.is_contiguous() and pb_index.numel() == times.numel()):
+        if not (isinstance(times, torch.Tensor) and times.device == dev and times.dtype is torch.float64
+                and times.is_contiguous()):
+            raise TypeError(f"times must be a contiguous {torch.float64} tensor on {dev}")
+        if not (isinstance(params, torch.Tensor) and params.device == dev and params.dtype is torch.float64
+                and params.is_contiguous()):
+            raise TypeError(f"params must be a contiguous {torch.float64} tensor on {dev}")
+        shape = params.shape
+        if len(shape) != 2 or shape[1] != self._nparam:
+            raise ValueError(f"params must have shape (npv, {self._nparam})")
+        npt = times.numel()
+        if pb_index is not None and not (pb_index.device == dev and pb_index.dtype is torch.int32
+                                         and pb_index.is_contiguous() and pb_index.numel() == npt):
             raise TypeError("pb_index must be a contiguous int32 tensor with one entry per time")
-        return times.numel(), params.shape[0]
+        return npt, shape[0]
+
+    def _cotangent(self, grad_flux, npv, npt):
+        if not (grad_flux.dtype is self.dtype and grad_flux.is_contiguous() and grad_flux.shape == (npv, npt)):
+            raise TypeError(f"grad_flux must be a contiguous {self.dtype} tensor of shape ({npv}, {npt})")
 
     def prepare(self, times: torch.Tensor, params: torch.Tensor, pb_index: Optional[torch.Tensor] = None,
                 supersampling=None, exptime=None, pv_status: Optional[torch.Tensor] = None,
@@ -321,15 +346,13 @@ class Model:
         Returns the workspace that holds the prepared batch; pass it as
         ``prepared=`` to both calls, with the same inputs."""
         npt, npv = self._inputs(times, params, pb_index)
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         if workspace is None:
             workspace = self.workspace(npv, npt, True)
-        st = self.lib.rr_prepare(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                                 ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                 ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _ptr(pv_status),
-                                 _ptr(workspace), workspace.numel(), _stream_handle(stream))
-        self._check(st)
+        st = self.lib.rr_prepare(self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp, exp_,
+                                 _ptr(pv_status), workspace.data_ptr(), workspace.numel(), _stream_handle(stream))
+        if st:
+            self._check(st)
         return workspace
 
     def evaluate(self, times: torch.Tensor, params: torch.Tensor, pb_index: Optional[torch.Tensor] = None,
@@ -340,8 +363,7 @@ class Model:
 
         prepared: a workspace filled by :meth:`prepare` with the same inputs."""
         npt, npv = self._inputs(times, params, pb_index)
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         if out is None:
             out = torch.empty((npv, npt), dtype=self.dtype, device=self.device)
         fn = self.lib.rr_evaluate
@@ -349,26 +371,39 @@ class Model:
             fn, workspace = self.lib.rr_evaluate_prepared, prepared
         elif workspace is None:
             workspace = self.workspace(npv, npt, False)
-        st = fn(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                _ptr(out), _ptr(pv_status), _ptr(workspace), workspace.numel(), _stream_handle(stream))
-        self._check(st)
+        st = fn(self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp, exp_, out.data_ptr(),
+                _ptr(pv_status), workspace.data_ptr(), workspace.numel(), _stream_handle(stream))
+        if st:
+            self._check(st)
         return out
+
+    def _prepare_and_evaluate(self, times, params, pb_index, supersampling, exptime):
+        """(flux, workspace): :meth:`prepare` and :meth:`evaluate` of it, with one look at the arguments."""
+        npt, npv = self._inputs(times, params, pb_index)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
+        workspace = self.workspace(npv, npt, True)
+        out = torch.empty((npv, npt), dtype=self.dtype, device=self.device)
+        head = (self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp, exp_)
+        tail = (workspace.data_ptr(), workspace.numel(), _stream_handle(None))
+        st = self.lib.rr_prepare(*head, None, *tail)
+        if st == 0:
+            st = self.lib.rr_evaluate_prepared(*head, out.data_ptr(), None, *tail)
+        if st:
+            self._check(st)
+        return out, workspace
 
     def evaluate_noalloc(self, times: torch.Tensor, params: torch.Tensor, pb_index: Optional[torch.Tensor] = None,
                          supersampling=None, exptime=None, out: Optional[torch.Tensor] = None,
                          pv_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         """As :meth:`evaluate`, with the library's fixed scratch instead of a workspace (see rr.h)."""
         npt, npv = self._inputs(times, params, pb_index)
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         if out is None:
             out = torch.empty((npv, npt), dtype=self.dtype, device=self.device)
-        st = self.lib.rr_evaluate_noalloc(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                                          ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                          ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _ptr(out),
-                                          _ptr(pv_status), _stream_handle(stream))
-        self._check(st)
+        st = self.lib.rr_evaluate_noalloc(self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp, exp_,
+                                          out.data_ptr(), _ptr(pv_status), _stream_handle(stream))
+        if st:
+            self._check(st)
         return out
 
     def evaluate_grad(self, times: torch.Tensor, params: torch.Tensor, grad_flux: torch.Tensor,
@@ -380,22 +415,19 @@ class Model:
 
         prepared: a workspace filled by :meth:`prepare` with the same inputs."""
         npt, npv = self._inputs(times, params, pb_index)
-        if not (grad_flux.dtype == self.dtype and grad_flux.is_contiguous() and grad_flux.shape == (npv, npt)):
-            raise TypeError(f"grad_flux must be a contiguous {self.dtype} tensor of shape ({npv}, {npt})")
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        self._cotangent(grad_flux, npv, npt)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         if out is None:
-            out = torch.empty((npv, self.nparam), dtype=torch.float64, device=self.device)
+            out = torch.empty((npv, self._nparam), dtype=torch.float64, device=self.device)
         fn = self.lib.rr_evaluate_grad
         if prepared is not None:
             fn, workspace = self.lib.rr_evaluate_grad_prepared, prepared
         elif workspace is None:
             workspace = self.workspace(npv, npt, True)
-        st = fn(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                _ptr(grad_flux), _ptr(out), _ptr(pv_status), _ptr(workspace), workspace.numel(),
-                _stream_handle(stream))
-        self._check(st)
+        st = fn(self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp, exp_, grad_flux.data_ptr(),
+                out.data_ptr(), _ptr(pv_status), workspace.data_ptr(), workspace.numel(), _stream_handle(stream))
+        if st:
+            self._check(st)
         return out
 
     def evaluate_both(self, times: torch.Tensor, params: torch.Tensor, grad_flux: torch.Tensor,
@@ -406,20 +438,18 @@ class Model:
         (rr_evaluate_both_prepared): the adjoint on a second stream of the context, beside the
         forward kernel; bitwise :meth:`evaluate` and :meth:`evaluate_grad` with ``prepared``."""
         npt, npv = self._inputs(times, params, pb_index)
-        if not (grad_flux.dtype == self.dtype and grad_flux.is_contiguous() and grad_flux.shape == (npv, npt)):
-            raise TypeError(f"grad_flux must be a contiguous {self.dtype} tensor of shape ({npv}, {npt})")
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        self._cotangent(grad_flux, npv, npt)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         if out is None:
             out = torch.empty((npv, npt), dtype=self.dtype, device=self.device)
         if grad_out is None:
-            grad_out = torch.empty((npv, self.nparam), dtype=torch.float64, device=self.device)
-        st = self.lib.rr_evaluate_both_prepared(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                                                ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                                ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                                                _ptr(grad_flux), _ptr(out), _ptr(grad_out), _ptr(pv_status),
-                                                _ptr(prepared), prepared.numel(), _stream_handle(stream))
-        self._check(st)
+            grad_out = torch.empty((npv, self._nparam), dtype=torch.float64, device=self.device)
+        st = self.lib.rr_evaluate_both_prepared(self._h, times.data_ptr(), _ptr(pb_index), npt, params.data_ptr(), npv, ssp,
+                                                exp_, grad_flux.data_ptr(), out.data_ptr(), grad_out.data_ptr(),
+                                                _ptr(pv_status), prepared.data_ptr(), prepared.numel(),
+                                                _stream_handle(stream))
+        if st:
+            self._check(st)
         return out, grad_out
 
     def evaluate_host(self, times, params, pb_index=None, supersampling=None, exptime=None, grad_flux=None,
@@ -462,13 +492,10 @@ class Model:
         f_h = result(out, (npv, npt), self.dtype)
         go_h = result(grad_out, (npv, nparam), torch.float64) if g_h is not None else None
         st_h = result(status_out, (npv,), torch.int32)
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
         with torch.cuda.device(self.device):
-            st = self.lib.rr_evaluate_host(self._h, _ptr(t_h), _ptr(pb_h), npt, _ptr(p_h), npv,
-                                           ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                           ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _ptr(g_h), _ptr(f_h),
-                                           _ptr(go_h), _ptr(st_h), int(chunk_pvs or 0))
+            st = self.lib.rr_evaluate_host(self._h, _ptr(t_h), _ptr(pb_h), npt, _ptr(p_h), npv, ssp, exp_, _ptr(g_h),
+                                           _ptr(f_h), _ptr(go_h), _ptr(st_h), int(chunk_pvs or 0))
         self._check(st)
         return f_h, go_h, st_h
 
@@ -483,12 +510,9 @@ class Model:
         All host tensors must be contiguous pinned CPU tensors of the model's
         types and stay untouched until the stream has passed the request."""
         npv, npt = int(params.shape[0]), int(times.numel())
-        ss = _host_array(supersampling, self.npb, np.int32, 1)
-        ex = _host_array(exptime, self.npb, np.float64, 0.0)
-        self._check(self.lib.rr_enqueue_host(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv,
-                                             ss.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                             ex.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _ptr(grad_flux),
-                                             _ptr(out), _ptr(grad_out), _ptr(status_out), _ptr(scratch),
+        ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
+        self._check(self.lib.rr_enqueue_host(self._h, _ptr(times), _ptr(pb_index), npt, _ptr(params), npv, ssp, exp_,
+                                             _ptr(grad_flux), _ptr(out), _ptr(grad_out), _ptr(status_out), _ptr(scratch),
                                              scratch.numel(), _stream_handle(stream)))
 
     def flux(self, times, params, pb_index=None, supersampling=None, exptime=None) -> torch.Tensor:
@@ -503,9 +527,12 @@ class _RRFlux(torch.autograd.Function):
         ctx.meta = (supersampling, exptime)
         p = params.detach()
         ctx.save_for_backward(times, pb_index, p)
+        if not params.requires_grad:
+            ctx.prepared = None
+            return model.evaluate(times, p, pb_index, supersampling, exptime)
         # one set-up for the forward and the backward pass, when a gradient is wanted
-        ctx.prepared = model.prepare(times, p, pb_index, supersampling, exptime) if params.requires_grad else None
-        return model.evaluate(times, p, pb_index, supersampling, exptime, prepared=ctx.prepared)
+        out, ctx.prepared = model._prepare_and_evaluate(times, p, pb_index, supersampling, exptime)
+        return out
 
     @staticmethod
     def backward(ctx, gflux):
