@@ -230,7 +230,9 @@ cudaError_t run_setup(rr_ctx* c, const double* times, const int32_t* pb_index, i
         return launch_pv_setup(c, params, npv, pbp, grad, ws, pv_status, s, times, pb_index, npt,
                                wb + W.pts_dt, wb + W.pts_pb, wb + W.pts_grp);
     });
-    if (e != cudaSuccess || c->cfg.npb == 1 || c->cfg.precision != RR_PREC_MIXED || npt == 0) return e;
+    if (e != cudaSuccess || npt == 0) return e;
+    // the chunk order, where a kernel of this record layout launches by it
+    if (!flux_ordered(c, npv, npt, grad) && !(grad && grad_ordered(c, npv, npt))) return e;
     return timed(c, RR_KERNEL_POINTS, s,
                  [&] { return launch_chunk_order(c, npt, wb + W.pts_grp, wb + W.pts_ord, s); });
 }

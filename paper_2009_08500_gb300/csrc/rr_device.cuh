@@ -262,7 +262,10 @@ __device__ __forceinline__ void half_angle_SV(float x, float& S, float& V) {
 // Newton step dx leaves an error of at most kepC dx^2 (kepC >= |f''/(2 f')|),
 // so the loop stops once that is below FP32 resolution of x; S and V follow x
 // by a first-order rotation, whose error dx^2 / 2 is below the same bound.
-// On return S = sin x, V = 1 - cos x.  Returns false if not converged.
+// On return S = sin x, V = 1 - cos x.  Returns false if not converged.  The
+// step's operations are spelled out, so that every kernel that inlines it rounds
+// alike (left to the compiler, x - dM was fused with the product that forms dM in one
+// instantiation and not in the others).
 __device__ __forceinline__ bool kepler_offset_f32(float dM, float ecE0, float esE0, float inv_den0, float kep2,
                                                   float kep3, float kepC, float& x, float& S, float& V, int& iters) {
     const float y = dM * inv_den0;
@@ -270,13 +273,13 @@ __device__ __forceinline__ bool kepler_offset_f32(float dM, float ecE0, float es
     #pragma unroll 1
     for (int it = 0; it < 24; ++it) {
         half_angle_SV(x, S, V);
-        const float fx = (x - dM) - ecE0 * S + esE0 * V;
-        const float fp = (1.0f - ecE0) + ecE0 * V + esE0 * S;
+        const float fx = fmaf(esE0, V, fmaf(-ecE0, S, __fsub_rn(x, dM)));
+        const float fp = fmaf(esE0, S, fmaf(ecE0, V, __fsub_rn(1.0f, ecE0)));
         const float dx = __fdividef(fx, fp);
         x -= dx;
         const float S_old = S;
-        S -= dx * (1.0f - V);
-        V -= dx * S_old;
+        S = fmaf(-dx, __fsub_rn(1.0f, V), S);
+        V = fmaf(-dx, S_old, V);
         iters = it + 1;
         if (kepC * dx * dx <= 1.5e-8f * fabsf(x) + 1e-37f) return true;
     }
@@ -1065,8 +1068,9 @@ struct GroupState {
     float Ah, Al, m;         // phase constants of pv `lane`
 };
 
-// Phase constants of the tile's pvs at the CTA's first group g0 (the only FP64
-// of the per-point kernels, once per CTA): cta_ph[i] = (A0h, A0l, m0, 0).
+// Phase constants of the tile's pvs at group g0, the first of the chunk of groups_per_cta(npt) groups that
+// the CTA belongs to (however finely the launch is cut, so that a phase does not depend on the
+// cut; the only FP64 of the per-point kernels, once per CTA): cta_ph[i] = (A0h, A0l, m0, 0).
 __device__ __forceinline__ void cta_phase(float4* cta_ph, const double* __restrict__ times, int g0,
                                           const char* recs, int rec_bytes, int npv_t) {
     for (int i = threadIdx.x; i < npv_t; i += blockDim.x) {
@@ -1094,14 +1098,13 @@ __device__ __forceinline__ void ff_sub(float ah, float al, float bh, float bl, f
 }
 
 // sg: the CTA's copy in shared memory of the summaries of its groups (sg[j]
-// for group gbeg + j, copied with the records); group gbeg is the phase
-// reference of cta_phase.  Plain loads (shared memory).
-__device__ __forceinline__ void group_load(GroupState& gs, const GroupInfo* sg, int j, const float4* cta_ph,
+// for group gbeg + j, copied with the records); t0: the offset (toff) of
+// cta_phase's reference group.  Plain loads (shared memory).
+__device__ __forceinline__ void group_load(GroupState& gs, const GroupInfo* sg, int j, float2 t0, const float4* cta_ph,
                                            const char* recs, int rec_bytes, int npv_t) {
     const int lane = threadIdx.x & 31;
     const float4 s0 = *reinterpret_cast<const float4*>(sg + j);
     const float2 tg = reinterpret_cast<const float2*>(sg + j)[2];
-    const float2 t0 = reinterpret_cast<const float2*>(sg)[2];
     gs.wlo = s0.x;
     gs.whi = s0.y;
     gs.maxdt = s0.z;

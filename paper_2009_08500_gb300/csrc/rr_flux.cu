@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
                                                                const int32_t* __restrict__ ppb,
                                                                const GroupInfo* __restrict__ grp,
                                                                int npt, int npv, PbParams pbp, RecLayout L,
-                                                               int pv_tile, int groups_per_cta,
+                                                               int pv_tile, int groups_per_cta, int chunk_groups,
                                                                const char* __restrict__ records,
                                                                const char* __restrict__ rowsg,
                                                                float* __restrict__ flux,
@@ -152,7 +152,9 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
     }
     if (__syncthreads_or(ok ? 0 : 1)) return;
     float4* cta_ph = reinterpret_cast<float4*>(smem + kOffCta);
-    cta_phase(cta_ph, times, gbeg, recs, L.head_bytes, npv_t);
+    const int gref = gbeg - gbeg % chunk_groups;
+    const float2 tref = __ldg(reinterpret_cast<const float2*>(grp + gref) + 2);   // its toff
+    cta_phase(cta_ph, times, gref, recs, L.head_bytes, npv_t);
     __syncthreads();
 
     const float nanf_ = __int_as_float(0x7fc00000);
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
     auto do_group = [&](int g) {
         const int p0 = g * kWarpPts + 4 * lane;
         GroupState gs;
-        group_load(gs, sgrp, g - gbeg, cta_ph, recs, L.head_bytes, npv_t);
+        group_load(gs, sgrp, g - gbeg, tref, cta_ph, recs, L.head_bytes, npv_t);
         unsigned bad;
         float4 cl;
         const unsigned may = group_decide(gs, recs, L.head_bytes, npv_t, bad, cl);
@@ -630,6 +632,27 @@ void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile) {
     while (pv_tile > 1 && ctas() < want) pv_tile = (pv_tile + 1) >> 1;
 }
 
+// The same for the FP32 kernels (gpc, pv_tile: the uncut launch's, kept from 3 CTAs per SM on): an
+// ensemble whose vectors transit together, or a few vectors, left most SMs without a CTA.  Pvs down to
+// 8 per CTA (an item per warp at least where every pv of the tile transits; 4 was slower) and parts of the
+// chunk (a multiple of 8 groups: a half, a quarter, an eighth, single groups), the forward kernel's groups
+// first, the adjoint's pvs first (its CTAs carry sums per (pv, group), and the finish kernel more partial
+// sums when the chunk is cut).  Measured, flux and adjoint: 16 pvs x 2,000 times 28.8 -> 11.8 and
+// 40.2 -> 13.9 us; 200 x 3,001 40.8 -> 12.8, 64.0 -> 19.4; 100 x 4,407 with 10 sub-exposures 69.1 ->
+// 13.5, 92.2 -> 17.5; 3 passbands, 256 x 9,001, adjoint 93.8 -> 35.2; prior populations 1,024 x 5,000
+// 24.9 -> 18.3, 33.1 -> 28.3.  With 6 CTAs per SM 1,024 x 5,000 takes 21.2 and 32.8, and tables staged
+// per CTA (256 pvs x 8 channels) 15.4 -> 18.3 from 4 on.
+void split32(const rr_ctx* c, int ngroups, int npv, bool adjoint, int& gpc, int& pv_tile) {
+    constexpr int min_tile = 8;
+    const long long want = 3LL * c->num_sms;
+    auto ctas = [&] { return (long long)((ngroups + gpc - 1) / gpc) * ((npv + pv_tile - 1) / pv_tile); };
+    auto cut_tile = [&] { while (pv_tile > min_tile && ctas() < want) pv_tile = (pv_tile + 1) >> 1; };
+    const int chunk = gpc;
+    if (adjoint) cut_tile();
+    while (gpc > 1 && ctas() < want) gpc = gpc * 8 > chunk ? gpc >> 1 : 1;
+    cut_tile();
+}
+
 // Failure-detection self-test: one bounded wait that nothing completes (see
 // rr_selftest_wait); the expiry is recorded in the error word like any other.
 __global__ void rr_selftest_kernel(int which, int* err) {
@@ -666,6 +689,40 @@ cudaError_t launch_selftest(rr_ctx* c, int which, cudaStream_t s) {
 // warp streams its groups first (heterogeneous workload: 835 -> 792 us).
 constexpr int kStreamWarpsSS1 = 2;
 
+// The cut of one forward launch.
+struct FluxCut {
+    int gpc, pv_tile, ngroups, per_pv;   // groups and pvs per CTA, groups, staged bytes per pv
+    bool stage_rows;   // FP32 kernel with several passbands: headers and rows of the tile in shared memory (the rows of
+                       // many passbands do not stay in L1); one passband, the adjoint's record layout (rows
+                       // 3 + nldc times larger) and the FP64 kernel: headers only, rows through L1/L2
+    bool q1;           // FP64: groups of 32 times
+    bool ordered;      // the time chunks are launched heaviest first
+};
+
+static FluxCut flux_cut(const rr_ctx* c, const RecLayout& L, int npv, int npt, bool grad_layout) {
+    const bool f64 = c->cfg.precision == RR_PREC_FP64;
+    FluxCut k;
+    k.stage_rows = !f64 && c->cfg.npb > 1 && !grad_layout;
+    k.per_pv = k.stage_rows ? L.head_bytes + L.rows_bytes : L.head_bytes;
+    k.pv_tile = pv_tile_for(k.per_pv);
+    k.gpc = groups_per_cta(npt);
+    k.ngroups = (npt + kWarpPts - 1) / kWarpPts;
+    // FP64, few (pv, group) pairs: groups of 32 times, so that an item is one pass of its warp
+    // (measured: 1 pv x 2,000 times 24.0 -> 13.8 us, 64 x 3,000 33.5 -> 29.4; 512 x 10,007 100 -> 96, but 200 x 5,000
+    // with 10 sub-exposures 180 -> 271: the candidates of 128 times fill a warp's passes better)
+    k.q1 = f64 && (long long)npv * k.ngroups < 16LL * c->num_sms;
+    if (k.q1) k.ngroups = (npt + 31) / 32;
+    if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
+    else split32(c, k.ngroups, npv, false, k.gpc, k.pv_tile);
+    k.ordered = !f64 && c->cfg.npb > 1 && k.gpc == groups_per_cta(npt) && k.ngroups > k.gpc;
+    return k;
+}
+
+bool flux_ordered(const rr_ctx* c, int npv, int npt, bool grad_layout) {
+    if (c->cfg.precision == RR_PREC_FP64) return false;
+    return flux_cut(c, make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout), npv, npt, grad_layout).ordered;
+}
+
 cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
@@ -673,22 +730,10 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
     const bool f64 = c->cfg.precision == RR_PREC_FP64;
     RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout)
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout);
-    // FP32 kernel with several passbands: headers and rows of the tile in
-    // shared memory (the rows of many passbands do not stay in L1); one
-    // passband, the adjoint's record layout (rows 3 + nldc times larger) and
-    // the FP64 kernel: headers only, rows through L1/L2
-    const bool stage_rows = !f64 && c->cfg.npb > 1 && !grad_layout;
-    const int per_pv = stage_rows ? L.head_bytes + L.rows_bytes : L.head_bytes;
-    int pv_tile = pv_tile_for(per_pv);
-    int gpc = groups_per_cta(npt);
-    int ngroups = (npt + kWarpPts - 1) / kWarpPts;
-    // FP64, few (pv, group) pairs: groups of 32 times, so that an item is one pass of its warp
-    // (measured: 1 pv x 2,000 times 24.0 -> 13.8 us, 64 x 3,000 33.5 -> 29.4; 512 x 10,007 100 -> 96, but 200 x 5,000
-    // with 10 sub-exposures 180 -> 271: the candidates of 128 times fill a warp's passes better)
-    const bool q1 = f64 && (long long)npv * ngroups < 16LL * c->num_sms;
-    if (q1) ngroups = (npt + 31) / 32;
-    if (f64) split64(c, ngroups, npv, gpc, pv_tile);
-    const size_t smem = flux_smem(pv_tile, per_pv, f64, gpc);
+    const FluxCut k = flux_cut(c, L, npv, npt, grad_layout);
+    const int pv_tile = k.pv_tile, gpc = k.gpc, ngroups = k.ngroups;
+    if (!k.ordered) pts_ord = nullptr;
+    const size_t smem = flux_smem(pv_tile, k.per_pv, f64, gpc);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
     const dim3 grid(npvt, (ngroups + gpc - 1) / gpc);
@@ -697,7 +742,7 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
     cudaError_t e;
     if (f64) {
-        auto kern = q1 ? (ss1 ? rr_flux_fp64_kernel<true, 1> : rr_flux_fp64_kernel<false, 1>)
+        auto kern = k.q1 ? (ss1 ? rr_flux_fp64_kernel<true, 1> : rr_flux_fp64_kernel<false, 1>)
                        : (ss1 ? rr_flux_fp64_kernel<true, 4> : rr_flux_fp64_kernel<false, 4>);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -706,11 +751,11 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
                                           (double*)flux, pv_status, bulk, c->d_err);
     } else {
         auto kern = c->counting
-                        ? (stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, true>
+                        ? (k.stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, true>
                                              : rr_flux_mixed_kernel<true, false, true>)
                                       : (ss1 ? rr_flux_mixed_kernel<false, true, true>
                                              : rr_flux_mixed_kernel<false, false, true>))
-                        : (stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, false>
+                        : (k.stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, false>
                                              : rr_flux_mixed_kernel<true, false, false>)
                                       : (ss1 ? rr_flux_mixed_kernel<false, true, false>
                                              : rr_flux_mixed_kernel<false, false, false>));
@@ -720,7 +765,8 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
         const int vec = (npt % 4 == 0) && (((uintptr_t)flux & 15u) == 0) ? (in_device_memory(flux) ? 3 : 1) : 0;
         kern<<<grid, kBlock, smem, s>>>(times, (const float2*)pts_dt, (const int32_t*)pts_pb,
                                         (const GroupInfo*)pts_grp, npt, npv, pbp, L,
-                                        pv_tile, gpc, (const char*)records, rowsg, (float*)flux, pv_status, vec,
+                                        pv_tile, gpc, groups_per_cta(npt), (const char*)records, rowsg, (float*)flux,
+                                        pv_status, vec,
                                         ss1 ? kStreamWarpsSS1 : (kBlock >> 5),
                                         c->d_counts ? c->d_counts + (size_t)RR_KERNEL_FLUX * RR_COUNT_KINDS : nullptr,
                                         (const int*)pts_ord, c->d_err);

@@ -304,9 +304,9 @@ template <bool DEP, bool SS1, bool COUNT>
 __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
     const double* __restrict__ times, const float2* __restrict__ pdt, const int32_t* __restrict__ ppb,
     const GroupInfo* __restrict__ grp, int npt,
-    int npv, PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta, const char* __restrict__ records,
-    const char* __restrict__ rowsg, const float* __restrict__ gflux, float* __restrict__ partials, int nacc,
-    int chromatic, int vec_g, const float4* __restrict__ svtab, unsigned long long* counts,
+    int npv, PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta, int chunk_groups,
+    const char* __restrict__ records, const char* __restrict__ rowsg, const float* __restrict__ gflux, float* __restrict__ partials, int nacc,
+    int chromatic, int vec_g, int pergroup, const float4* __restrict__ svtab, unsigned long long* counts,
     const int* __restrict__ chunk_order, int32_t* __restrict__ pv_status, int* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
     float* gacc = reinterpret_cast<float*>(recs + (size_t)pv_tile * L.head_bytes);   // [pv][group][nacc]
     float* depcols = gacc + (size_t)pv_tile * groups_per_cta * nacc;
     char* qbase = reinterpret_cast<char*>(depcols + (DEP ? (size_t)(nacc - 6) * kBlock : 0));
+    qbase += (16 - ((uint32_t)(qbase - (char*)smem) & 15u)) & 15u;   // the sums before it are of any length
     const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
     // the summaries of the CTA's groups, copied with the records, then the sine table of the
     // refinement (read by a lane alone, where an L2 read would hold its warp)
@@ -359,13 +360,15 @@ __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
     }
     if (__syncthreads_or(ok ? 0 : 1)) return;
     float4* cta_ph = reinterpret_cast<float4*>(smem + kOffCta);
-    cta_phase(cta_ph, times, gbeg, recs, L.head_bytes, npv_t);
+    const int gref = gbeg - gbeg % chunk_groups;
+    const float2 tref = __ldg(reinterpret_cast<const float2*>(grp + gref) + 2);   // its toff
+    cta_phase(cta_ph, times, gref, recs, L.head_bytes, npv_t);
     __syncthreads();
 
     // a group: the tile's transit mask -> work items
     auto do_group = [&](int g) {
         GroupState gs;
-        group_load(gs, sgrp, g - gbeg, cta_ph, recs, L.head_bytes, npv_t);
+        group_load(gs, sgrp, g - gbeg, tref, cta_ph, recs, L.head_bytes, npv_t);
         unsigned bad;
         float4 cl;
         const unsigned may = group_decide(gs, recs, L.head_bytes, npv_t, bad, cl);
@@ -518,7 +521,10 @@ __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
         __nanosleep(64);
     }
     if (COUNT) tally_flush(tl, counts);
-    cta_partials_groups<float>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, chunk, gridDim.y, partials);
+    if (pergroup)
+        cta_group_sums<float>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, gbeg, gend, ngroups, partials);
+    else
+        cta_partials_groups<float>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, chunk, gridDim.y, partials);
 }
 
 // FP64 form: the FP64 flux kernel's groups and items, each item's sums in its own (pv, group) slot as
@@ -795,8 +801,15 @@ static GradCut grad_cut(const rr_ctx* c, int npv, int npt) {
     };
     k.pv_tile = tile(k.gpc);
     if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
+    else split32(c, k.ngroups, npv, true, k.gpc, k.pv_tile);
     k.pergroup = k.gpc < k.chunk;
     return k;
+}
+
+bool grad_ordered(const rr_ctx* c, int npv, int npt) {
+    if (c->cfg.precision == RR_PREC_FP64 || c->cfg.npb == 1) return false;
+    const GradCut k = grad_cut(c, npv, npt);
+    return k.gpc == k.chunk && k.nchunks > 1;
 }
 
 size_t partials_bytes(const rr_ctx* c, int npv, int npt) {
@@ -827,6 +840,7 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     const size_t rsize = f64 ? 8 : 4;
     const GradCut k = grad_cut(c, npv, npt);
     const int pv_tile = k.pv_tile, gpc = k.gpc;
+    if (!grad_ordered(c, npv, npt)) pts_ord = nullptr;
     bool ss1 = true;
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
     const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1);
@@ -859,9 +873,9 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
         if (e != cudaSuccess) return e;                                                                      \
         KERNEL<<<grid, kBlock, smem, s>>>(times, (const float2*)pts_dt, (const int32_t*)pts_pb,                \
                                           (const GroupInfo*)pts_grp, npt, npv, pbp,                           \
-                                          L, pv_tile, gpc, (const char*)records, rowsg,                       \
+                                          L, pv_tile, gpc, k.chunk, (const char*)records, rowsg,              \
                                           (const float*)grad_flux, (float*)partials, nacc, c->cfg.chromatic,  \
-                                          vec_g, c->d_svtab, counts, (const int*)pts_ord,                     \
+                                          vec_g, k.pergroup, c->d_svtab, counts, (const int*)pts_ord,         \
                                           pv_status, c->d_err);                                               \
     } while (0)
         // bit 0: 16-byte loads; bit 1: L2 prefetches of cotangent rows (grad_flux in device memory)

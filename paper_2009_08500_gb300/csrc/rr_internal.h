@@ -326,6 +326,10 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
                         const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s);
+// whether the forward kernel (the records' layout) and the adjoint launch their time chunks heaviest first: several
+// passbands, several chunks, and a launch that is not cut below the chunk
+bool flux_ordered(const rr_ctx* c, int npv, int npt, bool grad_layout);
+bool grad_ordered(const rr_ctx* c, int npv, int npt);
 cudaError_t launch_chunk_order(rr_ctx* c, int npt, void* ws_grp, void* ws_ord, cudaStream_t s);
 // time chunks of the FP32 per-point kernels
 inline int time_chunks(int npt, int gpc) { return ((npt + kWarpPts - 1) / kWarpPts + gpc - 1) / gpc; }
@@ -385,4 +389,5 @@ void release_host_pipe(rr_ctx* c);
 int groups_per_cta(int npt);
 constexpr int kChunk64 = 8;   // 128-time groups per partial-sum chunk of the FP64 adjoint
 void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile);
+void split32(const rr_ctx* c, int ngroups, int npv, bool adjoint, int& gpc, int& pv_tile);
 }  // namespace rr
