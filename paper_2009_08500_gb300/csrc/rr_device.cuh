@@ -202,9 +202,29 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
     R h = (f1 * f2) * (f3 * f4);
     if (sizeof(R) == sizeof(float)) h = h > R(0) ? h : R(0);   // (the FP64 root takes negative h as 0)
     const R K = GRAD ? d_sqrt(h) : d_sqrt_sample(h);   // the adjoint keeps the rounding-exact root
-    const R zz = z * z, kk = k * k;
-    const R kap0 = d_atan2(K, zz + (one - kk));
-    const R kap1 = d_atan2(K, zz + (kk - one));
+    R zz, kk, x0, x1, kap0, kap1;
+    if constexpr (sizeof(R) == sizeof(float)) {   // spelled out: the same rounding in every instantiation
+        zz = __fmul_rn(z, z);
+        kk = __fmul_rn(k, k);
+        x0 = __fadd_rn(zz, __fsub_rn(one, kk));
+        x1 = __fadd_rn(zz, __fsub_rn(kk, one));
+    } else {
+        zz = z * z;
+        kk = k * k;
+        x0 = zz + (one - kk);
+        x1 = zz + (kk - one);
+    }
+    bool usual = false;
+    if constexpr (!GRAD && sizeof(R) == sizeof(float)) usual = k > 1e-3f && k < 0.69f;
+    if (usual) {
+        // tan kappa_0 <= k / sqrt(1 - k^2) < 1, and of K and |x1| the larger is at least 1.4 k z: less
+        // folding, the same values (heterogeneous series 461 -> 450 us; no gain in the adjoint)
+        kap0 = atan2_upper((float)K, (float)x0, true);
+        kap1 = atan2_upper((float)K, (float)x1, false, true);
+    } else {
+        kap0 = d_atan2(K, x0);
+        kap1 = d_atan2(K, x1);
+    }
     if (GRAD) {
         dAdz = -K * d_rcp(z);
         dAdk = R(2) * k * kap1;

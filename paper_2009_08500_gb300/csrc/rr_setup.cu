@@ -546,8 +546,7 @@ __global__ void __launch_bounds__(kDirWarps * 32) rr_direct_table_kernel(
 // together (a thread per node left 30% of the lanes idle), nodes are numbered
 // through the rows, edges and profiles come from shared memory, and the parts of
 // edge_area that no lane of a warp needs (the closed forms outside the lens, the
-// small-angle series or the arctangent form, the compensated factors when
-// c >= 2k) are skipped by warp votes.  Bound by instruction issue (79% of the
+// small-angle series, the compensated factors when c >= 2k) are skipped.  Bound by instruction issue (79% of the
 // slots, 31.6 of 32 lanes).  Measured against a thread per node, quadratic law, 200 +
 // 300 annuli, 200 nodes: 1,000 pvs 328 -> 156 us (with dT/dk 339 -> 170), 16 pvs
 // 117 -> 33; 2,048 pvs 552 -> 338 with dT/dk and shared weights; nonlinear law (five
@@ -559,7 +558,7 @@ constexpr int kDirNodes = kDirCta / kDirLanes;          // nodes per CTA
 constexpr size_t kDirSmem = 48 * 1024;                  // most shared memory of a CTA
 constexpr int kDirMinNz = 48;                           // fewest annuli
 
-// edge_area for a whole warp: the same operations, with votes in place of selects where the warp agrees.
+// edge_area for a whole warp: the same operations, with branches in place of selects where warps mostly agree.
 // FAR: every lane's node has c >= 2k; in the lens then sin kappa_0 <= k / c <= 1/2, so that angle lies below
 // the diagonal and its segment in the range of the series.
 template <bool FAR>
@@ -584,24 +583,24 @@ __device__ __forceinline__ float edge_area_warp(float r, float k, float c, float
     const float drk = r - k;
     const float x0 = fabsf(drk) < fabsf(c - k) ? fmaf(drk, r + k, c2) : fmaf(c - k, c + k, r2);
     const float x1 = fabsf(drk) < fabsf(c - r) ? fmaf(-drk, r + k, c2) : fmaf(c - r, c + r, k2);
-    const float kap1 = atan2_upper(K, x1, false, FAR);
     const float q = K * inv4c2;
-    float seg0;
+    float seg0, kap0, kap1;
     if (FAR) {
-        seg0 = __fmul_rn(r2, seg_phi_small(atan2_upper(K, x0, true)));
-    } else {
-        const float kap0 = atan2_upper(K, x0);
+        kap0 = atan2_upper(K, x0, true);
+        kap1 = atan2_upper(K, x1, false, true);
         seg0 = __fmul_rn(r2, seg_phi_small(kap0));
-        if (__any_sync(0xffffffffu, !(kap0 < 0.75f)))
-            if (!(kap0 < 0.75f)) seg0 = fmaf(r2, kap0, -__fmul_rn(q, x0));
+    } else {
+        kap0 = atan2_upper(K, x0);
+        kap1 = atan2_upper(K, x1);
+        seg0 = __fmul_rn(r2, seg_phi_small(kap0));
+        if (!(kap0 < 0.75f)) seg0 = fmaf(r2, kap0, -__fmul_rn(q, x0));
     }
     float seg1 = fmaf(k2, kap1, -__fmul_rn(q, x1));
-    if (__any_sync(0xffffffffu, kap1 < 0.75f))
-        if (kap1 < 0.75f) seg1 = __fmul_rn(k2, seg_phi_small(kap1));
+    if (kap1 < 0.75f) seg1 = __fmul_rn(k2, seg_phi_small(kap1));
     float a = __fadd_rn(seg0, seg1);
     float ddk = __fmul_rn(__fmul_rn(2.0f, k), kap1), ddc = __fmul_rn(-K, inv_c);
     // disjoint and nested circles: one of the vanishing factors, and with it P, is not positive
-    if (__any_sync(0xffffffffu, !lens)) {
+    if (!lens) {
         if (s2 <= 0.0f) { a = CUDART_PI_F * r2; ddk = 0.0f; ddc = 0.0f; }
         if (p2 <= 0.0f) { a = CUDART_PI_F * k2; ddk = 2.0f * CUDART_PI_F * k; ddc = 0.0f; }
         if (p1 <= 0.0f) { a = 0.0f; ddk = 0.0f; ddc = 0.0f; }
