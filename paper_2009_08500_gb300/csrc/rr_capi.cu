@@ -232,7 +232,7 @@ cudaError_t run_setup(rr_ctx* c, const double* times, const int32_t* pb_index, i
     });
     if (e != cudaSuccess || npt == 0) return e;
     // the chunk order, where a kernel of this record layout launches by it
-    if (!flux_ordered(c, npv, npt, grad) && !(grad && grad_ordered(c, npv, npt))) return e;
+    if (!flux_ordered(c, pbp, npv, npt, grad) && !(grad && grad_ordered(c, pbp, npv, npt))) return e;
     return timed(c, RR_KERNEL_POINTS, s,
                  [&] { return launch_chunk_order(c, npt, wb + W.pts_grp, wb + W.pts_ord, s); });
 }

@@ -696,7 +696,7 @@ struct FluxCut {
                        // many passbands do not stay in L1); one passband, the adjoint's record layout (rows
                        // 3 + nldc times larger) and the FP64 kernel: headers only, rows through L1/L2
     bool q1;           // FP64: groups of 32 times
-    bool ordered;      // the time chunks are launched heaviest first
+    bool uncut;        // FP32: several whole chunks (they may be launched heaviest first)
 };
 
 static FluxCut flux_cut(const rr_ctx* c, const RecLayout& L, int npv, int npt, bool grad_layout) {
@@ -714,13 +714,13 @@ static FluxCut flux_cut(const rr_ctx* c, const RecLayout& L, int npv, int npt, b
     if (k.q1) k.ngroups = (npt + 31) / 32;
     if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
     else split32(c, k.ngroups, npv, false, k.gpc, k.pv_tile);
-    k.ordered = !f64 && c->cfg.npb > 1 && k.gpc == groups_per_cta(npt) && k.ngroups > k.gpc;
+    k.uncut = !f64 && k.gpc == groups_per_cta(npt) && k.ngroups > k.gpc;
     return k;
 }
 
-bool flux_ordered(const rr_ctx* c, int npv, int npt, bool grad_layout) {
-    if (c->cfg.precision == RR_PREC_FP64) return false;
-    return flux_cut(c, make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout), npv, npt, grad_layout).ordered;
+bool flux_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt, bool grad_layout) {
+    if (c->cfg.precision == RR_PREC_FP64 || !mixed_sampling(pbp)) return false;
+    return flux_cut(c, make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout), npv, npt, grad_layout).uncut;
 }
 
 cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
@@ -732,7 +732,7 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, grad_layout);
     const FluxCut k = flux_cut(c, L, npv, npt, grad_layout);
     const int pv_tile = k.pv_tile, gpc = k.gpc, ngroups = k.ngroups;
-    if (!k.ordered) pts_ord = nullptr;
+    if (!k.uncut || !mixed_sampling(pbp)) pts_ord = nullptr;
     const size_t smem = flux_smem(pv_tile, k.per_pv, f64, gpc);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;

@@ -806,8 +806,8 @@ static GradCut grad_cut(const rr_ctx* c, int npv, int npt) {
     return k;
 }
 
-bool grad_ordered(const rr_ctx* c, int npv, int npt) {
-    if (c->cfg.precision == RR_PREC_FP64 || c->cfg.npb == 1) return false;
+bool grad_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt) {
+    if (c->cfg.precision == RR_PREC_FP64 || !mixed_sampling(pbp)) return false;
     const GradCut k = grad_cut(c, npv, npt);
     return k.gpc == k.chunk && k.nchunks > 1;
 }
@@ -840,7 +840,7 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     const size_t rsize = f64 ? 8 : 4;
     const GradCut k = grad_cut(c, npv, npt);
     const int pv_tile = k.pv_tile, gpc = k.gpc;
-    if (!grad_ordered(c, npv, npt)) pts_ord = nullptr;
+    if (!grad_ordered(c, pbp, npv, npt)) pts_ord = nullptr;
     bool ss1 = true;
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
     const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1);

@@ -326,10 +326,15 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
                         const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s);
-// whether the forward kernel (the records' layout) and the adjoint launch their time chunks heaviest first: several
-// passbands, several chunks, and a launch that is not cut below the chunk
-bool flux_ordered(const rr_ctx* c, int npv, int npt, bool grad_layout);
-bool grad_ordered(const rr_ctx* c, int npv, int npt);
+// whether the forward kernel (the records' layout) and the adjoint launch their time chunks heaviest first:
+// passbands of different supersampling, several chunks, and a launch that is not cut below the chunk
+bool flux_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt, bool grad_layout);
+bool grad_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt);
+inline bool mixed_sampling(const PbParams& pbp) {
+    for (int pb = 1; pb < pbp.npb; ++pb)
+        if (pbp.ss[pb] != pbp.ss[0]) return true;
+    return false;
+}
 cudaError_t launch_chunk_order(rr_ctx* c, int npt, void* ws_grp, void* ws_ord, cudaStream_t s);
 // time chunks of the FP32 per-point kernels
 inline int time_chunks(int npt, int gpc) { return ((npt + kWarpPts - 1) / kWarpPts + gpc - 1) / gpc; }

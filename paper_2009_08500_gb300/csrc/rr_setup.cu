@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kDirWarps * 32) rr_direct_table_kernel(
 constexpr int kDirLanes = 4;
 constexpr int kDirCta = 128;                             // threads per CTA
 constexpr int kDirNodes = kDirCta / kDirLanes;          // nodes per CTA
-constexpr size_t kDirSmem = 48 * 1024;                  // most shared memory of a CTA
+constexpr size_t kDirSmem = 48 * 1024 - kDirNodes * sizeof(double);   // most dynamic shared memory of a CTA
 constexpr int kDirMinNz = 48;                           // fewest annuli
 
 // edge_area for a whole warp: the same operations, with branches in place of selects where warps mostly agree.
@@ -635,6 +635,7 @@ __global__ void __launch_bounds__(kDirCta, 1024 / kDirCta) rr_direct_lanes_kerne
         const float* __restrict__ basis, const double* __restrict__ basis64, const float* __restrict__ pre,
         const float* __restrict__ pre_lo, DirectTables D) {
     extern __shared__ float dsh[];
+    __shared__ double kd_s[kDirNodes];             // the weights' radius ratio of the CTA's rows, -1: invalid
     const int ng = mp.ng, nz = mp.nz, nb_all = mp.nbasis;
     const int lane = threadIdx.x & 31, sub = lane % kDirLanes;
     float* ze = dsh;                               // nz + 1 edges
@@ -645,38 +646,47 @@ __global__ void __launch_bounds__(kDirCta, 1024 / kDirCta) rr_direct_lanes_kerne
         for (int j = threadIdx.x; j < nz; j += blockDim.x)
             lb[((size_t)(b / kDirLanes) * nz + j) * kDirLanes + b % kDirLanes] =
                 b < nb_all ? __ldg(basis + (size_t)b * nz + j) : 0.0f;
-    __syncthreads();
     const int nkp = mp.chromatic ? mp.npb : 1;
     const int rpp = mp.shared ? 1 : nkp;   // rows per pv
+    const long long first = (long long)blockIdx.x * kDirNodes;
+    const int row0 = (int)(first / ng);
+    const int off0 = (int)(first - (long long)row0 * ng);
+    // the radius ratios once per CTA (FP64: the mean of 8 channels in every warp took as long as a tenth of the
+    // edges' arithmetic)
+    for (int r = threadIdx.x; r <= (off0 + kDirNodes - 1) / ng && row0 + r < D.nrows; r += blockDim.x) {
+        const int pv = (row0 + r) / rpp;
+        const double* ks = params + (size_t)pv * mp.nparam + 6;
+        double kd;
+        if (mp.shared) {
+            // the mean of the pv's per-passband radius ratios (invalid if any is)
+            kd = 0.0;
+            bool ok = true;
+            for (int j = 0; j < nkp; ++j) {
+                const double kj = ks[j];
+                ok = ok && kj > 0.0 && kj < 1.0;
+                kd += kj;
+            }
+            kd = ok ? kd / nkp : -1.0;
+        } else {
+            kd = ks[row0 + r - pv * rpp];
+        }
+        // (rows of small-planet passbands are not read: their rows come from the profile directly)
+        kd_s[r] = kd > 0.0 && kd < 1.0 && !(kd < mp.k_small) ? kd : -1.0;
+    }
+    __syncthreads();
     const bool own = mp.ld_model == RR_LD_TABULATED && mp.chromatic && !mp.shared;   // a row: its passband's table only
     float* Thi = reinterpret_cast<float*>(D.hi);
     float* Tdk = reinterpret_cast<float*>(D.dk);
     const size_t bstride = (size_t)D.nrows * ng;
     const int src = lane & ~(kDirLanes - 1);       // the node's first lane
-    const long long first = (long long)blockIdx.x * kDirNodes;
-    const int row0 = (int)(first / ng);
-    const int off = (int)(first - (long long)row0 * ng) + threadIdx.x / kDirLanes;
-    int row = row0 + off / ng;
-    const int ig = off % ng;
+    const int off = off0 + threadIdx.x / kDirLanes;
+    const int ig = off % ng, row = row0 + off / ng;
     const bool live = row < D.nrows;
     if (!__any_sync(0xffffffffu, live)) return;
-    row = live ? row : D.nrows - 1;
-    const int pv = row / rpp, slot = row - pv * rpp;
-    double kd;
-    if (mp.shared) {
-        kd = 0.0;
-        bool ok = true;
-        for (int j = 0; j < nkp; ++j) {
-            const double kj = params[(size_t)pv * mp.nparam + 6 + j];
-            ok = ok && kj > 0.0 && kj < 1.0;
-            kd += kj;
-        }
-        kd = ok ? kd / nkp : -1.0;
-    } else {
-        kd = params[(size_t)pv * mp.nparam + 6 + slot];
-    }
+    const int slot = row % rpp;
+    const double kd = live ? kd_s[off / ng] : -1.0;
     const size_t o = (size_t)row * ng + ig;
-    const bool valid = live && kd > 0.0 && kd < 1.0 && !(kd < mp.k_small);
+    const bool valid = __double2hiint(kd) >= 0;   // kd > 0
     const float k = (float)kd;
     const double gd = ig * mp.dg;
     const double cd = gd * (1.0 + (double)k);
@@ -1059,10 +1069,12 @@ __device__ __forceinline__ void table_rows(const ModelParams& mp, const RecLayou
 }
 
 // ... and direct model: the pv's own projections (row ik of the per-call tables); the in-cell slopes come from
-// the differences of the FP32 pairs.
-template <typename R>
-__device__ __forceinline__ void direct_rows(const ModelParams& mp, const RecLayout& L, const DirectTables& D, int grad, R* r0,
-                                            int ig, int b0, int ik, int nc, const R (&uc)[4], const R (&Ic)[4], R invIs) {
+// the differences of the FP32 pairs.  The passbands pb .. pb_end - 1 that share the row (one radius ratio, or
+// shared weights; a named law) are written from one set of loads: of(pb) sets their row block, coefficients
+// and 1 / I_star.
+template <typename R, typename F>
+__device__ __forceinline__ void direct_rows(const ModelParams& mp, const RecLayout& L, const DirectTables& D, int grad, int ig,
+                                            int b0, int ik, int nc, const R (&Ic)[4], int pb, int pb_end, F&& of) {
     using V = RowVec<R>;
     constexpr int N = V::N;
     const int ng = mp.ng;
@@ -1072,60 +1084,78 @@ __device__ __forceinline__ void direct_rows(const ModelParams& mp, const RecLayo
     const float* Lp = N == 4 ? D.lo + o0 : nullptr;   // the lo parts exist in the FP32 form
     const R* Kp = grad ? reinterpret_cast<const R*>(D.dk) + o0 : nullptr;
     const bool last = ig + N >= ng;
-    V v, dv, kv;
+    V vb[5], dd[5], kk[5];   // per basis: the projections, their differences to the next node, d / dk
     #pragma unroll
     for (int c = 0; c < 5; ++c) {
         if (c == 0 || c <= nc) {
-            const R w = c == 0 ? R(1) : uc[c - 1];
             const V h = V::load(Hp + c * ds);
             V l;
             if constexpr (N == 4) l = V::load(Lp + c * ds);
             #pragma unroll
-            for (int q = 0; q < N; ++q) {
-                const R vb = N == 4 ? h.v[q] + l.v[q] : h.v[q];
-                v.v[q] = c == 0 ? vb : v.v[q] + w * vb;
-            }
+            for (int q = 0; q < N; ++q) vb[c].v[q] = N == 4 ? h.v[q] + l.v[q] : h.v[q];
             if (grad) {
                 const R hn = last ? R(0) : Hp[c * ds + N];
                 R ln = R(0);
                 if constexpr (N == 4) ln = last ? R(0) : Lp[c * ds + N];
-                const V k = V::load(Kp + c * ds);
+                kk[c] = V::load(Kp + c * ds);
                 #pragma unroll
                 for (int q = 0; q < N; ++q) {
-                    R dd = (q < N - 1 ? h.v[q < N - 1 ? q + 1 : q] : hn) - h.v[q];
-                    if (N == 4) dd += (q < N - 1 ? l.v[q < N - 1 ? q + 1 : q] : ln) - l.v[q];
-                    if (q < N - 1 || !last) dv.v[q] += w * dd;
-                    kv.v[q] += w * k.v[q];
+                    dd[c].v[q] = (q < N - 1 ? h.v[q < N - 1 ? q + 1 : q] : hn) - h.v[q];
+                    if (N == 4) dd[c].v[q] += (q < N - 1 ? l.v[q < N - 1 ? q + 1 : q] : ln) - l.v[q];
                 }
             }
         }
     }
-    V ldw;
-    #pragma unroll
-    for (int q = 0; q < N; ++q) ldw.v[q] = v.v[q] * invIs;
-    ldw.store(r0 + ig);
-    if (!grad) return;
-    V o;
-    #pragma unroll
-    for (int q = 0; q < N; ++q) o.v[q] = dv.v[q] * invIs;
-    o.store(r0 + L.ng_pad + ig);
-    #pragma unroll
-    for (int q = 0; q < N; ++q) o.v[q] = kv.v[q] * invIs;
-    o.store(r0 + 2 * L.ng_pad + ig);
-    #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        if (c < nc) {
-            const V h = V::load(Hp + (1 + c) * ds);
-            V l;
-            if constexpr (N == 4) l = V::load(Lp + (1 + c) * ds);
-            #pragma unroll
-            for (int q = 0; q < N; ++q) {
-                const R vb = N == 4 ? h.v[q] + l.v[q] : h.v[q];
-                o.v[q] = (vb - ldw.v[q] * Ic[c]) * invIs;
+    #pragma unroll 1
+    for (; pb < pb_end; ++pb) {
+        R uc[4], invIs;
+        R* r0 = of(pb, uc, invIs);
+        V ldw, o, v = vb[0];
+        #pragma unroll
+        for (int c = 1; c < 5; ++c) {
+            if (c <= nc) {
+                #pragma unroll
+                for (int q = 0; q < N; ++q) v.v[q] += uc[c - 1] * vb[c].v[q];
             }
-            o.store(r0 + (size_t)(3 + c) * L.ng_pad + ig);
+        }
+        #pragma unroll
+        for (int q = 0; q < N; ++q) ldw.v[q] = v.v[q] * invIs;
+        ldw.store(r0 + ig);
+        if (!grad) continue;
+        V dv, kv;
+        #pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            if (c == 0 || c <= nc) {
+                const R w = c == 0 ? R(1) : uc[c - 1];
+                #pragma unroll
+                for (int q = 0; q < N; ++q) {
+                    if (q < N - 1 || !last) dv.v[q] += w * dd[c].v[q];
+                    kv.v[q] += w * kk[c].v[q];
+                }
+            }
+        }
+        #pragma unroll
+        for (int q = 0; q < N; ++q) o.v[q] = dv.v[q] * invIs;
+        o.store(r0 + L.ng_pad + ig);
+        #pragma unroll
+        for (int q = 0; q < N; ++q) o.v[q] = kv.v[q] * invIs;
+        o.store(r0 + 2 * L.ng_pad + ig);
+        #pragma unroll
+        for (int c = 1; c < 5; ++c) {
+            if (c <= nc) {
+                #pragma unroll
+                for (int q = 0; q < N; ++q) o.v[q] = (vb[c].v[q] - ldw.v[q] * Ic[c - 1]) * invIs;
+                o.store(r0 + (size_t)(2 + c) * L.ng_pad + ig);
+            }
         }
     }
+}
+
+// Direct model of a named affine law whose passbands all take the pv's one row (vector units of rr_pv_setup_kernel;
+// a pv below k_small is, with every passband, a small-planet row and not shared).
+__host__ __device__ inline bool rows_shared(const ModelParams& mp) {
+    return mp.direct && mp.npb > 1 && (mp.shared || !mp.chromatic) && mp.k_small == 0.0 &&
+           mp.ld_model != RR_LD_TABULATED && mp.ld_model != RR_LD_POWER2 && mp.ld_model != RR_LD_POWER2_PM;
 }
 
 // The launch has three kinds of CTAs, independent of each other: the per-time preparation (two
@@ -1147,8 +1177,9 @@ constexpr int kHeadWinThreads = 128;
 // 2 per CTA, measured 49.7 -> 39.6 us for 2,048 pvs; 1 per CTA was slower again), and fewer while the
 // launch leaves SMs without a CTA.
 constexpr int kRowPvs = 8;
+// (4 where one unit of a warp writes all passbands).
 static int row_pvs_per_cta(const rr_ctx* c, int npv) {
-    int n = c->cfg.npb >= 4 ? 2 : (c->cfg.npb >= 2 ? 4 : kRowPvs);
+    int n = c->cfg.npb >= 4 ? (rows_shared(model_params(c)) ? 4 : 2) : (c->cfg.npb >= 2 ? 4 : kRowPvs);
     while (n > 1 && (npv + n - 1) / n < 2 * c->num_sms) n >>= 1;
     return n;
 }
@@ -1595,11 +1626,14 @@ __global__ void __launch_bounds__(256, 4) rr_pv_setup_kernel(ModelParams mp, PbP
     const bool vec = mp.ng % NV == 0;
     const int span = vec ? 32 * NV : 64;
     const int nchunk = (L.ng_pad + span - 1) / span;
-    const int nunits = nloc * mp.npb * nchunk;
+    // direct model, the passbands of a pv share its row: one unit for all of them
+    const bool share = vec && rows_shared(mp);
+    const int upb = share ? 1 : mp.npb;   // units per pv and span
+    const int nunits = nloc * upb * nchunk;
     #pragma unroll 1
     for (int w = tid >> 5; w < nunits; w += blockDim.x >> 5) {
         const int rw = w / nchunk, ch = w - rw * nchunk;
-        const int lp = rw / mp.npb, pb = rw - lp * mp.npb;
+        const int lp = rw / upb, pb = rw - lp * upb;
         if (st_s[lp] != 0) continue;
         R* r0 = reinterpret_cast<R*>(rows_region + (size_t)(pv0 + lp) * L.rows_bytes) +
                 (size_t)pb * L.rows_per_pb * L.ng_pad;
@@ -1709,9 +1743,15 @@ __global__ void __launch_bounds__(256, 4) rr_pv_setup_kernel(ModelParams mp, PbP
             const int ig = span * ch + lane * NV;
             if (ig < L.ng_pad) {
                 if (ig >= mp.ng) {
-                    for (int r = 0; r < L.rows_per_pb; ++r) RowVec<R>{}.store(r0 + (size_t)r * L.ng_pad + ig);
+                    for (int r = 0; r < L.rows_per_pb * (share ? mp.npb : 1); ++r) RowVec<R>{}.store(r0 + (size_t)r * L.ng_pad + ig);
                 } else if (mp.direct) {
-                    direct_rows<R>(mp, L, D, grad, r0, ig, b0, ik, nc, uc, Ic, invIs);
+                    direct_rows<R>(mp, L, D, grad, ig, b0, ik, nc, Ic, pb, share ? mp.npb : pb + 1,
+                                   [&](int p, R (&u)[4], R& iIs) {
+                                       #pragma unroll
+                                       for (int c = 0; c < 4; ++c) u[c] = c < nc ? u_s[lp][p][c] : R(0);
+                                       iIs = invIs_s[lp][p];
+                                       return r0 + (size_t)(p - pb) * L.rows_per_pb * L.ng_pad;
+                                   });
                 } else {
                     table_rows<R>(mp, L, T, DT, grad, r0, ig, b0, ik, nc, uc, Ic, ak, bk, invIs, inv_dk);
                 }
