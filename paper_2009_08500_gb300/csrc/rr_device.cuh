@@ -185,10 +185,10 @@ __device__ __forceinline__ double d_rcp(double x) { return div64(1.0, x); }
 // The contact factors f1 = 1 + k - z (outer contact) and f3 = z - (1 - k)
 // (inner contact) are arguments: the mixed adjoint passes them from FP64 near
 // the contacts, where K ~ sqrt(f1 f3) amplifies their rounding.
-template <typename R, bool GRAD>
+template <typename R, bool GRAD, bool LENS = false>
 __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& dAdk) {
     const R one = R(1);
-    if (z <= fabs(one - k)) {
+    if (!LENS && z <= fabs(one - k)) {
         if (GRAD) dAdz = R(0);
         if (k < one) {
             if (GRAD) dAdk = R(2) * Tr<R>::pi() * k;
@@ -232,9 +232,9 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
     return kap0 + kk * kap1 - R(0.5) * K;
 }
 
-template <typename R, bool GRAD>
+template <typename R, bool GRAD, bool LENS = false>
 __device__ __forceinline__ R covered_area(R k, R z, R& dAdz, R& dAdk) {
-    return covered_area_f13<R, GRAD>(k, z, (R(1) + k) - z, z - (R(1) - k), dAdz, dAdk);
+    return covered_area_f13<R, GRAD, LENS>(k, z, (R(1) + k) - z, z - (R(1) - k), dAdz, dAdk);
 }
 
 // Linear interpolation of a profile row over the g nodes g_i = i / (ng - 1):
@@ -255,19 +255,22 @@ __device__ __forceinline__ R lerp_row(const R* row, int ng, R g, R& slope_cell, 
 
 // S = sin x and V = 1 - cos x for |x| <= 1 from their Taylor series in x^2
 // (through x^9 and x^10: truncation below 3e-8 of S and 5e-9 of V), V
-// without cancellation; larger |x| from the half angle.
+// without cancellation; half_angle_SV takes larger |x| from the half angle.
+__device__ __forceinline__ void small_angle_SV(float x, float& S, float& V) {
+    const float x2 = x * x;
+    float ps = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);    // 1/9!, -1/7!
+    ps = fmaf(x2, ps, 8.3333333e-3f);                       // 1/5!
+    ps = fmaf(x2, ps, -1.6666667e-1f);                      // -1/3!
+    S = fmaf(x * x2, ps, x);
+    float pv = fmaf(x2, 2.7557319e-7f, -2.4801587e-5f);    // 1/10!, -1/8!
+    pv = fmaf(x2, pv, 1.3888889e-3f);                       // 1/6!
+    pv = fmaf(x2, pv, -4.1666668e-2f);                      // -1/4!
+    pv = fmaf(x2, pv, 0.5f);                                // 1/2!
+    V = x2 * pv;
+}
 __device__ __forceinline__ void half_angle_SV(float x, float& S, float& V) {
     if (fabsf(x) <= 1.0f) {
-        const float x2 = x * x;
-        float ps = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);    // 1/9!, -1/7!
-        ps = fmaf(x2, ps, 8.3333333e-3f);                       // 1/5!
-        ps = fmaf(x2, ps, -1.6666667e-1f);                      // -1/3!
-        S = fmaf(x * x2, ps, x);
-        float pv = fmaf(x2, 2.7557319e-7f, -2.4801587e-5f);    // 1/10!, -1/8!
-        pv = fmaf(x2, pv, 1.3888889e-3f);                       // 1/6!
-        pv = fmaf(x2, pv, -4.1666668e-2f);                      // -1/4!
-        pv = fmaf(x2, pv, 0.5f);                                // 1/2!
-        V = x2 * pv;
+        small_angle_SV(x, S, V);
     } else {
         float hs, hc;
         sincosf(0.5f * x, &hs, &hc);
@@ -302,6 +305,39 @@ __device__ __forceinline__ bool kepler_offset_f32(float dM, float ecE0, float es
         V = fmaf(-dx, S_old, V);
         iters = it + 1;
         if (kepC * dx * dx <= 1.5e-8f * fabsf(x) + 1e-37f) return true;
+    }
+    return false;
+}
+
+// The forward kernel's solve: the same equation, start and series with a step of third order
+// (Chebyshev's, d = dx + f''/(2 f') dx^2 with Newton's dx = f / f') and S, V turned by d to second order.
+// A step leaves at most (2 kepC^2 + kepC / 3) |dx|^3 (the third derivative's share is below kepC / 3), so nearly every
+// sample is done after one where one in 25 of Newton's needed two, and with it nearly every warp.
+__device__ __forceinline__ bool kepler_step3_f32(float dM, const float4 ke, float kepC, float& x, float& S, float& V) {
+    const float ec = ke.y, es = ke.z, C = __fsub_rn(1.0f, V);
+    const float f = fmaf(es, V, fmaf(-ec, S, __fsub_rn(x, dM)));
+    const float fp = fmaf(es, S, fmaf(-ec, C, 1.0f));
+    const float f2 = fmaf(es, C, ec * S);
+    const float r = div_normal(1.0f, fp);
+    const float dx = f * r, dx2 = dx * dx;
+    const float d = fmaf(0.5f * f2 * r, dx2, dx), h = 0.5f * d * d;
+    const float S_old = S;
+    x -= d;
+    S = fmaf(-h, S_old, fmaf(-d, C, S_old));
+    V = fmaf(h, C, fmaf(-d, S_old, V));
+    return kepC * fmaf(2.0f, kepC, 1.0f / 3.0f) * dx2 * fabsf(dx) <= fmaf(1.5e-8f, fabsf(x), 1e-37f);
+}
+__device__ __forceinline__ float kepler_start_f32(float dM, const float4 ke, const float4 ks) {
+    const float y = dM * ke.w;
+    return fmaf(fmaf(ks.z, y, ks.y), y * y, y);
+}
+__device__ __forceinline__ bool kepler_offset3_f32(float dM, const float4 ke, const float4 ks, float& x, float& S, float& V,
+                                                   int& iters) {
+    x = kepler_start_f32(dM, ke, ks);
+    #pragma unroll 1
+    for (iters = 1; iters <= 24; ++iters) {
+        half_angle_SV(x, S, V);
+        if (kepler_step3_f32(dM, ke, ks.w, x, S, V)) return true;
     }
     return false;
 }
@@ -529,7 +565,8 @@ __device__ __forceinline__ Orbit32 orbit32(const PvHead<float>& H, float dM, dou
     } else {
         const float4 ke = quad(H.e);        // e, ecE0, esE0, inv_den0
         const float4 ks = quad(H.wmax_c);   // wmax_c, kep2, kep3, kepC
-        o.ok = kepler_offset_f32(dM, ke.y, ke.z, ke.w, ks.y, ks.z, ks.w, x, o.S, o.V, iters);
+        if (APPROX_Z) o.ok = kepler_offset3_f32(dM, ke, ks, x, o.S, o.V, iters);
+        else o.ok = kepler_offset_f32(dM, ke.y, ke.z, ke.w, ks.y, ks.z, ks.w, x, o.S, o.V, iters);
     }
     o.x = x;
     const float4 ax = quad(H.ax1);          // ax1, ax2, ay1, ay2
@@ -1033,6 +1070,12 @@ __device__ __forceinline__ void tally_flush(const Tally& t, unsigned long long* 
     }
 }
 
+// Mean-anomaly offset of sub-exposure s (an exact integer) of a time at phase fr_h + fr_l (cycles).
+__device__ __forceinline__ float sample_dM(const PvHead<float>& H, float fr_h, float fr_l, float s, float first, float step) {
+    const float x = __fadd_rn(fmaf(fmaf(s, step, first), H.Bh, fr_h), fr_l);
+    return __fmul_rn(6.28318530717958647692f, __fsub_rn(x, round_nearest(x)));
+}
+
 // One sub-exposure of one (pv, time): delta = A Ib (Eq. 5 without the 1 -),
 // 0 outside the transit.  Kepler failure: bad = true, NaN.  COUNT: add the
 // sample's work to `tl`.
@@ -1041,13 +1084,11 @@ __device__ __forceinline__ float delta32(const PvHead<float>& H, const PvPb<floa
                                          int ng, float fr_h, float fr_l, float s, float first, float step, bool& bad,
                                          Tally* tl = nullptr) {
     if (COUNT) ++tl->n[RR_COUNT_SAMPLES];
-    const float off = fmaf(s, step, first) * H.Bh;   // sub-exposure s (exact integer), offset in cycles
-    float x = (fr_h + off) + fr_l;
-    x -= round_nearest(x);
-    const float dM = 6.28318530717958647692f * x;
+    const float dM = sample_dM(H, fr_h, fr_l, s, first, step);
     if (fabsf(dM) > pbc.win_s) return 0.0f;
     double dMd = 0.0;
     if (H.flags & kPvKepler64) {
+        const float off = fmaf(s, step, first) * H.Bh;
         double xd = ((double)fr_h + (double)off) + (double)fr_l;
         xd -= rint(xd);
         dMd = 6.283185307179586476925 * xd;
@@ -1074,6 +1115,99 @@ __device__ __forceinline__ float delta32(const PvHead<float>& H, const PvPb<floa
     int cell;
     const float A = covered_area<float, false>(pq.x, o.z, d0, d1);
     return A * lerp_row<float>(row, ng, g, sl, cell);
+}
+
+// A sub-exposure's place: its time's phase (cycles), index, passband constants, sub-exposure spacing, profile row.
+struct Sub32 {
+    float2 fr;
+    float s;
+    float first, step;
+    const PvPb<float>* pbc;
+    const float* row;
+};
+
+// Two sub-exposures of one pv at once (delta32 of each, the same bits).  The supersampled forward kernel
+// is bound by instructions issued, and in small launches by the chain of a sample: a pair reads the
+// header once, has two independent chains, and is straight code up to the lens area.  two: whether
+// there is a second one.  What the straight form does not take (FP64 orbits, a second step of the
+// Kepler solve, |x| > 1) goes through delta32, one after the other.  Measured, flux kernel with one
+// sample per step and Newton's steps / pairs and third-order steps: 2,048 pvs x 60,000 times with 1, 10
+// and 30 sub-exposures 450 / 406 us, 128 x 20,000 53 / 37, 256 x 9,001 (1, 5, 10) 29 / 25, one pv x
+// 19,440 (10) 26.8 / 20.6.  Three CTAs per SM (no spills) in place of four: 461.
+__device__ __forceinline__ void delta32_pair(const PvHead<float>& H, const Sub32 (&a)[2], bool two, int ng, float (&d)[2], bool& bad) {
+    const int flags = H.flags;
+    float dM[2], x[2], S[2], V[2];
+    bool in[2];
+    #pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        d[i] = 0.0f;
+        dM[i] = sample_dM(H, a[i].fr.x, a[i].fr.y, a[i].s, a[i].first, a[i].step);
+        in[i] = !(fabsf(dM[i]) > a[i].pbc->win_s) && (i == 0 || two);
+        if (!in[i]) dM[i] = 0.0f;
+    }
+    if (!in[0] && !in[1]) return;
+    bool straight = !(flags & kPvKepler64);
+    if (flags & kPvCircular) {
+        #pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            straight &= fabsf(dM[i]) <= 1.0f;
+            small_angle_SV(dM[i], S[i], V[i]);
+        }
+    } else {
+        const float4 ke = quad(H.e);        // e, ecE0, esE0, inv_den0
+        const float4 ks = quad(H.wmax_c);   // wmax_c, kep2, kep3, kepC
+        #pragma unroll
+        for (int i = 0; i < 2; ++i) {       // kepler_offset3_f32's start and first step
+            x[i] = kepler_start_f32(dM[i], ke, ks);
+            straight &= fabsf(x[i]) <= 1.0f;
+            small_angle_SV(x[i], S[i], V[i]);
+            straight &= kepler_step3_f32(dM[i], ke, ks.w, x[i], S[i], V[i]);
+        }
+    }
+    if (!straight) {
+        #pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+            const bool f = i == 0;
+            if (!(f ? in[0] : in[1])) continue;
+            const float r = delta32<false>(H, f ? *a[0].pbc : *a[1].pbc, f ? a[0].row : a[1].row, ng, f ? a[0].fr.x : a[1].fr.x,
+                                           f ? a[0].fr.y : a[1].fr.y, f ? a[0].s : a[1].s, f ? a[0].first : a[1].first,
+                                           f ? a[0].step : a[1].step, bad);
+            if (f) d[0] = r; else d[1] = r;
+        }
+        return;
+    }
+    const float4 ax = quad(H.ax1);          // ax1, ax2, ay1, ay2
+    const float4 ab = quad(H.a);            // a, b, a2, b2
+    const float rho0 = H.rho0;
+    float z[2], k[2], A[2], I[2];
+    bool lens = false;
+    #pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float Px = fmaf(ax.x, V[i], ax.y * S[i]);
+        const float Py = rho0 + fmaf(ax.z, V[i], ax.w * S[i]);
+        z[i] = sqrt_approx(fmaf(ab.z * Px, Px, ab.w * Py * Py));
+        const float2 pq = *reinterpret_cast<const float2*>(&a[i].pbc->k);   // k, inv1pk
+        k[i] = pq.x;
+        const float g = z[i] * pq.y;
+        in[i] = in[i] && Py > 0.0f && !(g >= 1.0f);
+        A[i] = Tr<float>::pi() * k[i] * k[i];
+        if (!(k[i] < 1.0f)) A[i] = Tr<float>::pi();
+        lens |= in[i] && !(z[i] <= fabsf(1.0f - k[i]));
+        float sl;
+        int cell;
+        I[i] = lerp_row<float>(a[i].row, ng, in[i] ? g : 0.0f, sl, cell);
+    }
+    if (lens) {
+        #pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float d0, d1;
+            const float Al = covered_area<float, false, true>(k[i], z[i], d0, d1);
+            if (!(z[i] <= fabsf(1.0f - k[i]))) A[i] = Al;
+        }
+    }
+    #pragma unroll
+    for (int i = 0; i < 2; ++i)
+        if (in[i]) d[i] = A[i] * I[i];
 }
 
 

@@ -280,22 +280,56 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
                 float sub = (float)(e_beg - (pw >> 5));
                 float part = 0.0f;
                 jh = j;
-                #pragma unroll 1
-                for (int e = e_beg; e < e_end; ++e) {
-                    if (e == next) {
-                        // candidate j ends inside the run: the head's sum, or a final one
-                        if (j == jh) ph = part; else wl->pacc[j] = part;
-                        ++j;
-                        pw = wl->ps[j];
-                        next = wl->ps[j + 1] >> 5;
-                        pb = pw & 31;
-                        cd = wl->cand[j];
-                        sub = 0.0f;
-                        part = 0.0f;
+                const size_t row_stride = (size_t)L.rows_per_pb * L.ng_pad;
+                if constexpr (COUNT) {   // one sample at a time
+                    #pragma unroll 1
+                    for (int e = e_beg; e < e_end; ++e) {
+                        if (e == next) {
+                            // candidate j ends inside the run: the head's sum, or a final one
+                            if (j == jh) ph = part; else wl->pacc[j] = part;
+                            ++j;
+                            pw = wl->ps[j];
+                            next = wl->ps[j + 1] >> 5;
+                            pb = pw & 31;
+                            cd = wl->cand[j];
+                            sub = 0.0f;
+                            part = 0.0f;
+                        }
+                        part += delta32<COUNT>(H, PB[pb], rows + pb * row_stride, L.ng, cd.x, cd.y,
+                                               sub, ps->first[pb], ps->step[pb], bad, &tl);
+                        sub += 1.0f;
                     }
-                    part += delta32<COUNT>(H, PB[pb], rows + (size_t)pb * L.rows_per_pb * L.ng_pad, L.ng, cd.x, cd.y,
-                                           sub, ps->first[pb], ps->step[pb], bad, &tl);
-                    sub += 1.0f;
+                } else {   // two at a time, the second possibly of the next candidate
+                    #pragma unroll 1
+                    for (int e = e_beg; e < e_end; e += 2) {
+                        auto finish = [&]() {   // candidate j ends inside the run: the head's sum, or a final one
+                            if (j == jh) ph = part; else wl->pacc[j] = part;
+                            ++j;
+                            next = wl->ps[j + 1] >> 5;
+                            part = 0.0f;
+                        };
+                        if (e == next) {
+                            finish();
+                            pb = wl->ps[j] & 31;
+                            cd = wl->cand[j];
+                            sub = 0.0f;
+                        }
+                        const bool two = e + 1 < e_end, cross = two && e + 1 == next;
+                        Sub32 a[2];
+                        a[0] = {cd, sub, ps->first[pb], ps->step[pb], PB + pb, rows + pb * row_stride};
+                        if (cross) {
+                            pb = wl->ps[j + 1] & 31;
+                            cd = wl->cand[j + 1];
+                            sub = -1.0f;
+                        }
+                        a[1] = {cd, sub + 1.0f, ps->first[pb], ps->step[pb], PB + pb, rows + pb * row_stride};
+                        float d[2];
+                        delta32_pair(H, a, two, L.ng, d, bad);
+                        part += d[0];
+                        if (cross) finish();
+                        part += d[1];
+                        sub += 2.0f;
+                    }
                 }
                 if (j == jh) ph = part; else { jt = j; pt = part; }
             }
