@@ -176,6 +176,9 @@ __device__ __forceinline__ float d_rcp(float x) {
 }
 __device__ __forceinline__ double d_rcp(double x) { return div64(1.0, x); }
 
+// Radius ratios whose half-angles need less folding (covered_area_f13).
+__device__ __forceinline__ bool usual_k(float k) { return k > 1e-3f && k < 0.69f; }
+
 // Area covered by a planet of radius k at centre distance z on a unit stellar
 // disk (the a(c, k) of Eq. 5), for z < 1 + k, with its partial derivatives.
 // Lens case: A = kappa0 + k^2 kappa1 - K/2 with K = sqrt of Heron's product
@@ -184,7 +187,8 @@ __device__ __forceinline__ double d_rcp(double x) { return div64(1.0, x); }
 // common chord), dA/dk = 2 k kappa1 (planet rim inside the star).
 // The contact factors f1 = 1 + k - z (outer contact) and f3 = z - (1 - k)
 // (inner contact) are arguments: the mixed adjoint passes them from FP64 near
-// the contacts, where K ~ sqrt(f1 f3) amplifies their rounding.
+// the contacts, where K ~ sqrt(f1 f3) amplifies their rounding.  LENS: the planet is known to
+// cross the limb and k to be a usual_k.
 template <typename R, bool GRAD, bool LENS = false>
 __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& dAdk) {
     const R one = R(1);
@@ -214,8 +218,8 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
         x0 = zz + (one - kk);
         x1 = zz + (kk - one);
     }
-    bool usual = false;
-    if constexpr (!GRAD && sizeof(R) == sizeof(float)) usual = k > 1e-3f && k < 0.69f;
+    bool usual = LENS;
+    if constexpr (!LENS && !GRAD && sizeof(R) == sizeof(float)) usual = usual_k(k);
     if (usual) {
         // tan kappa_0 <= k / sqrt(1 - k^2) < 1, and of K and |x1| the larger is at least 1.4 k z: less
         // folding, the same values (heterogeneous series 461 -> 450 us; no gain in the adjoint)
@@ -229,6 +233,7 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
         dAdz = -K * d_rcp(z);
         dAdk = R(2) * k * kap1;
     }
+    if constexpr (sizeof(R) == sizeof(float)) return fmaf(-0.5f, K, fmaf(kk, kap1, kap0));
     return kap0 + kk * kap1 - R(0.5) * K;
 }
 
@@ -546,7 +551,7 @@ __device__ __forceinline__ float4 quad(const float& first) { return *reinterpret
 // rounding reaches the flux with a factor below 1); the adjoint takes the
 // rounding-exact one, since near a contact point its z-derivative amplifies
 // z's rounding by 1 / (2 (1 + k - z)).
-template <bool APPROX_Z = true>
+template <bool APPROX_Z = true, bool K64 = true>
 __device__ __forceinline__ Orbit32 orbit32(const PvHead<float>& H, float dM, double dMd, int& iters) {
     Orbit32 o;
     o.ok = true;
@@ -556,7 +561,7 @@ __device__ __forceinline__ Orbit32 orbit32(const PvHead<float>& H, float dM, dou
     if (flags & kPvCircular) {
         half_angle_SV(dM, o.S, o.V);
         x = dM;
-    } else if (flags & kPvKepler64) {
+    } else if (K64 && (flags & kPvKepler64)) {
         double xd, Sd, Vd;
         o.ok = kepler_offset_f64(dMd, H.ecE0d, H.esE0d, H.inv_den0d, xd, Sd, Vd);
         o.S = (float)Sd;
@@ -1076,25 +1081,12 @@ __device__ __forceinline__ float sample_dM(const PvHead<float>& H, float fr_h, f
     return __fmul_rn(6.28318530717958647692f, __fsub_rn(x, round_nearest(x)));
 }
 
-// One sub-exposure of one (pv, time): delta = A Ib (Eq. 5 without the 1 -),
-// 0 outside the transit.  Kepler failure: bad = true, NaN.  COUNT: add the
-// sample's work to `tl`.
-template <bool COUNT = false>
-__device__ __forceinline__ float delta32(const PvHead<float>& H, const PvPb<float>& pbc, const float* __restrict__ row,
-                                         int ng, float fr_h, float fr_l, float s, float first, float step, bool& bad,
-                                         Tally* tl = nullptr) {
-    if (COUNT) ++tl->n[RR_COUNT_SAMPLES];
-    const float dM = sample_dM(H, fr_h, fr_l, s, first, step);
-    if (fabsf(dM) > pbc.win_s) return 0.0f;
-    double dMd = 0.0;
-    if (H.flags & kPvKepler64) {
-        const float off = fmaf(s, step, first) * H.Bh;
-        double xd = ((double)fr_h + (double)off) + (double)fr_l;
-        xd -= rint(xd);
-        dMd = 6.283185307179586476925 * xd;
-    }
+// delta32 from the mean-anomaly offset dM inside the window (dMd: the same in FP64).
+template <bool COUNT, bool K64 = true>
+__device__ __forceinline__ float delta32_at(const PvHead<float>& H, const PvPb<float>& pbc, const float* __restrict__ row,
+                                            int ng, float dM, double dMd, bool& bad, Tally* tl = nullptr) {
     int iters;
-    const Orbit32 o = orbit32(H, dM, dMd, iters);
+    const Orbit32 o = orbit32<true, K64>(H, dM, dMd, iters);
     if (COUNT) {
         ++tl->n[RR_COUNT_ORBIT];
         if (H.flags & kPvCircular) ++tl->n[RR_COUNT_CIRCULAR];
@@ -1114,7 +1106,27 @@ __device__ __forceinline__ float delta32(const PvHead<float>& H, const PvPb<floa
     float d0, d1, sl;
     int cell;
     const float A = covered_area<float, false>(pq.x, o.z, d0, d1);
-    return A * lerp_row<float>(row, ng, g, sl, cell);
+    return __fmul_rn(A, lerp_row<float>(row, ng, g, sl, cell));
+}
+
+// One sub-exposure of one (pv, time): delta = A Ib (Eq. 5 without the 1 -),
+// 0 outside the transit.  Kepler failure: bad = true, NaN.  COUNT: add the
+// sample's work to `tl`.
+template <bool COUNT = false>
+__device__ __forceinline__ float delta32(const PvHead<float>& H, const PvPb<float>& pbc, const float* __restrict__ row,
+                                         int ng, float fr_h, float fr_l, float s, float first, float step, bool& bad,
+                                         Tally* tl = nullptr) {
+    if (COUNT) ++tl->n[RR_COUNT_SAMPLES];
+    const float dM = sample_dM(H, fr_h, fr_l, s, first, step);
+    if (fabsf(dM) > pbc.win_s) return 0.0f;
+    double dMd = 0.0;
+    if (H.flags & kPvKepler64) {
+        const float off = fmaf(s, step, first) * H.Bh;
+        double xd = ((double)fr_h + (double)off) + (double)fr_l;
+        xd -= rint(xd);
+        dMd = 6.283185307179586476925 * xd;
+    }
+    return delta32_at<COUNT>(H, pbc, row, ng, dM, dMd, bad, tl);
 }
 
 // A sub-exposure's place: its time's phase (cycles), index, passband constants, sub-exposure spacing, profile row.
@@ -1129,24 +1141,37 @@ struct Sub32 {
 // Two sub-exposures of one pv at once (delta32 of each, the same bits).  The supersampled forward kernel
 // is bound by instructions issued, and in small launches by the chain of a sample: a pair reads the
 // header once, has two independent chains, and is straight code up to the lens area.  two: whether
-// there is a second one.  What the straight form does not take (FP64 orbits, a second step of the
-// Kepler solve, |x| > 1) goes through delta32, one after the other.  Measured, flux kernel with one
-// sample per step and Newton's steps / pairs and third-order steps: 2,048 pvs x 60,000 times with 1, 10
-// and 30 sub-exposures 450 / 406 us, 128 x 20,000 53 / 37, 256 x 9,001 (1, 5, 10) 29 / 25, one pv x
-// 19,440 (10) 26.8 / 20.6.  Three CTAs per SM (no spills) in place of four: 461.
+// there is a second one.  What the straight form does not take goes through delta32, one after the other:
+// FP64 orbits and unusual radius ratios at once, a second step of the Kepler solve and |x| > 1 from the
+// anomaly on.  Samples outside the window are not branched around: a warp has hardly ever none inside.
+// Measured, flux kernel with one sample per step and Newton's steps / pairs and third-order steps:
+// 2,048 pvs x 60,000 times with 1, 10 and 30 sub-exposures 450 / 394 us, 128 x 20,000 53 / 34, 256 x
+// 9,001 (1, 5, 10) 29 / 24.5, one pv x 19,440 (10) 26.8 / 18.8.  Three CTAs per SM in place of four: 434.
 __device__ __forceinline__ void delta32_pair(const PvHead<float>& H, const Sub32 (&a)[2], bool two, int ng, float (&d)[2], bool& bad) {
+    d[0] = d[1] = 0.0f;
     const int flags = H.flags;
+    const float4 q0 = quad(a[0].pbc->k), q1 = quad(a[1].pbc->k);   // k, inv1pk, win_s, win_p
+    const float k[2] = {q0.x, q1.x}, inv1pk[2] = {q0.y, q1.y}, win_s[2] = {q0.z, q1.z};
+    if ((flags & kPvKepler64) || !usual_k(k[0]) || !usual_k(k[1])) {
+        #pragma unroll 1
+        for (int i = 0; i < (two ? 2 : 1); ++i) {
+            const bool f = i == 0;
+            const float r = delta32<false>(H, f ? *a[0].pbc : *a[1].pbc, f ? a[0].row : a[1].row, ng, f ? a[0].fr.x : a[1].fr.x,
+                                           f ? a[0].fr.y : a[1].fr.y, f ? a[0].s : a[1].s, f ? a[0].first : a[1].first,
+                                           f ? a[0].step : a[1].step, bad);
+            if (f) d[0] = r; else d[1] = r;
+        }
+        return;
+    }
     float dM[2], x[2], S[2], V[2];
     bool in[2];
     #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        d[i] = 0.0f;
         dM[i] = sample_dM(H, a[i].fr.x, a[i].fr.y, a[i].s, a[i].first, a[i].step);
-        in[i] = !(fabsf(dM[i]) > a[i].pbc->win_s) && (i == 0 || two);
+        in[i] = !(fabsf(dM[i]) > win_s[i]) && (i == 0 || two);
         if (!in[i]) dM[i] = 0.0f;
     }
-    if (!in[0] && !in[1]) return;
-    bool straight = !(flags & kPvKepler64);
+    bool straight = true;
     if (flags & kPvCircular) {
         #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -1169,9 +1194,8 @@ __device__ __forceinline__ void delta32_pair(const PvHead<float>& H, const Sub32
         for (int i = 0; i < 2; ++i) {
             const bool f = i == 0;
             if (!(f ? in[0] : in[1])) continue;
-            const float r = delta32<false>(H, f ? *a[0].pbc : *a[1].pbc, f ? a[0].row : a[1].row, ng, f ? a[0].fr.x : a[1].fr.x,
-                                           f ? a[0].fr.y : a[1].fr.y, f ? a[0].s : a[1].s, f ? a[0].first : a[1].first,
-                                           f ? a[0].step : a[1].step, bad);
+            const float r = delta32_at<false, false>(H, f ? *a[0].pbc : *a[1].pbc, f ? a[0].row : a[1].row, ng,
+                                                     f ? dM[0] : dM[1], 0.0, bad);
             if (f) d[0] = r; else d[1] = r;
         }
         return;
@@ -1179,35 +1203,32 @@ __device__ __forceinline__ void delta32_pair(const PvHead<float>& H, const Sub32
     const float4 ax = quad(H.ax1);          // ax1, ax2, ay1, ay2
     const float4 ab = quad(H.a);            // a, b, a2, b2
     const float rho0 = H.rho0;
-    float z[2], k[2], A[2], I[2];
+    float z[2], A[2], I[2];
     bool lens = false;
     #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const float Px = fmaf(ax.x, V[i], ax.y * S[i]);
         const float Py = rho0 + fmaf(ax.z, V[i], ax.w * S[i]);
         z[i] = sqrt_approx(fmaf(ab.z * Px, Px, ab.w * Py * Py));
-        const float2 pq = *reinterpret_cast<const float2*>(&a[i].pbc->k);   // k, inv1pk
-        k[i] = pq.x;
-        const float g = z[i] * pq.y;
+        const float g = z[i] * inv1pk[i];
         in[i] = in[i] && Py > 0.0f && !(g >= 1.0f);
         A[i] = Tr<float>::pi() * k[i] * k[i];
-        if (!(k[i] < 1.0f)) A[i] = Tr<float>::pi();
-        lens |= in[i] && !(z[i] <= fabsf(1.0f - k[i]));
+        lens |= in[i] && !(z[i] <= 1.0f - k[i]);
         float sl;
         int cell;
-        I[i] = lerp_row<float>(a[i].row, ng, in[i] ? g : 0.0f, sl, cell);
+        I[i] = lerp_row<float>(a[i].row, ng, g, sl, cell);   // (its cell is in range for any g >= 0)
     }
     if (lens) {
         #pragma unroll
         for (int i = 0; i < 2; ++i) {
             float d0, d1;
             const float Al = covered_area<float, false, true>(k[i], z[i], d0, d1);
-            if (!(z[i] <= fabsf(1.0f - k[i]))) A[i] = Al;
+            if (!(z[i] <= 1.0f - k[i])) A[i] = Al;
         }
     }
     #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (in[i]) d[i] = A[i] * I[i];
+        if (in[i]) d[i] = __fmul_rn(A[i], I[i]);   // (rounded before it is summed, as delta32's)
 }
 
 
