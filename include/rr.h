@@ -288,7 +288,9 @@ rr_status rr_evaluate_grad_prepared(rr_ctx* ctx, const double* times, const int3
  * rr_evaluate_prepared and rr_evaluate_grad_prepared in one call, the adjoint
  * on a second stream of the context that forks from `stream` and joins it
  * again, so that the adjoint (latency-bound) runs beside the forward kernel
- * (an output stream).  Arguments as the two calls; flux and grad_params both
+ * (an output stream).  In the FP64 form with one sample per time one kernel
+ * on `stream` writes both (profiled as RR_KERNEL_GRAD): an orbit and an area
+ * serve both results.  Arguments as the two calls; flux and grad_params both
  * written; results bitwise those of the two calls.  The paper has no
  * counterpart.  The context's second stream is created on first use and
  * freed by rr_destroy; like every entry point, calls on one context must not

@@ -281,7 +281,7 @@ rr_status evaluate_impl(rr_ctx* c, const double* times, const int32_t* pb_index,
 rr_status evaluate_grad_impl(rr_ctx* c, const double* times, const int32_t* pb_index, int32_t npt,
                              const double* params, int32_t npv, const int32_t* ss, const double* exptime,
                              const void* grad_flux, double* grad_params, int32_t* pv_status, void* ws,
-                             size_t ws_bytes, bool prepared, void* stream) {
+                             size_t ws_bytes, bool prepared, void* stream, void* flux = nullptr) {
     PbParams pbp;
     rr_status st = check_eval(c, times, pb_index, npt, params, npv, ss, exptime, grad_params, ws, ws_bytes, true, pbp);
     if (st != RR_OK) return st;
@@ -305,7 +305,7 @@ rr_status evaluate_grad_impl(rr_ctx* c, const double* times, const int32_t* pb_i
     if ((e = timed(c, RR_KERNEL_GRAD, s, [&] {
              return launch_grad(c, times, pb_index, wb + W.pts_dt, wb + W.pts_pb, wb + W.pts_grp,
                                 c->cfg.npb > 1 ? wb + W.pts_ord : nullptr, npt, npv, pbp, ws, grad_flux, partials,
-                                pv_status, s);
+                                pv_status, s, flux);
          })) != cudaSuccess)
         return cuda_fail(c, e, "adjoint kernel");
     if ((e = timed(c, RR_KERNEL_GRAD_REDUCE, s, [&] {
@@ -561,6 +561,10 @@ rr_status rr_evaluate_both_prepared(rr_ctx* c, const double* times, const int32_
     NvtxRange nvtx_range("rr_evaluate_both_prepared");
     if (!c) return fail(nullptr, RR_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
+    // FP64 form, one sample per time: one kernel for both
+    if (flux && grad_with_flux(c, ss, npv, npt))
+        return evaluate_grad_impl(c, times, pb_index, npt, params, npv, ss, exptime, grad_flux, grad_params, pv_status,
+                                  const_cast<void*>(ws), ws_bytes, true, stream, flux);
     cudaError_t e = cudaSetDevice(c->cfg.device);
     if (e == cudaSuccess && !c->aux) e = cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking);
     if (e == cudaSuccess && !c->ev_fork) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);

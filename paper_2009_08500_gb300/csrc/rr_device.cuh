@@ -206,17 +206,16 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
     R h = (f1 * f2) * (f3 * f4);
     if (sizeof(R) == sizeof(float)) h = h > R(0) ? h : R(0);   // (the FP64 root takes negative h as 0)
     const R K = GRAD ? d_sqrt(h) : d_sqrt_sample(h);   // the adjoint keeps the rounding-exact root
-    R zz, kk, x0, x1, kap0, kap1;
+    R kk, x0, x1, kap0, kap1;
     if constexpr (sizeof(R) == sizeof(float)) {   // spelled out: the same rounding in every instantiation
-        zz = __fmul_rn(z, z);
+        const R zz = __fmul_rn(z, z);
         kk = __fmul_rn(k, k);
         x0 = __fadd_rn(zz, __fsub_rn(one, kk));
         x1 = __fadd_rn(zz, __fsub_rn(kk, one));
     } else {
-        zz = z * z;
-        kk = k * k;
-        x0 = zz + (one - kk);
-        x1 = zz + (kk - one);
+        kk = __dmul_rn(k, k);
+        x0 = fma(z, z, __dsub_rn(one, kk));
+        x1 = fma(z, z, __dsub_rn(kk, one));
     }
     bool usual = LENS;
     if constexpr (!LENS && !GRAD && sizeof(R) == sizeof(float)) usual = usual_k(k);
@@ -233,8 +232,7 @@ __device__ __forceinline__ R covered_area_f13(R k, R z, R f1, R f3, R& dAdz, R& 
         dAdz = -K * d_rcp(z);
         dAdk = R(2) * k * kap1;
     }
-    if constexpr (sizeof(R) == sizeof(float)) return fmaf(-0.5f, K, fmaf(kk, kap1, kap0));
-    return kap0 + kk * kap1 - R(0.5) * K;
+    return fma(R(-0.5), K, fma(kk, kap1, kap0));
 }
 
 template <typename R, bool GRAD, bool LENS = false>
@@ -247,7 +245,8 @@ __device__ __forceinline__ R covered_area(R k, R z, R& dAdz, R& dAdk) {
 // the in-cell slope d/dg.
 template <typename R>
 __device__ __forceinline__ R lerp_row(const R* row, int ng, R g, R& slope_cell, int& cell) {
-    const R x = g * R(ng - 1);
+    R x;
+    if constexpr (sizeof(R) == sizeof(double)) x = __dmul_rn(g, R(ng - 1)); else x = g * R(ng - 1);
     int i = (int)x;                       // x >= 0: truncation is floor
     i = i < ng - 2 ? i : ng - 2;
     const R al = x - R(i);
@@ -1817,5 +1816,74 @@ constexpr size_t kOff64Wl = kOff64Pb + sizeof(PbShared64);
 constexpr int kBlock64 = 64;   // threads per CTA
 constexpr size_t kOff64Recs = kOff64Wl + (kBlock64 / 32) * kList64Bytes;
 static_assert(kOff64Wl % 16 == 0 && kOff64Recs % 16 == 0, "16-byte regions");
+
+// One sample: A Ib (Eq. 5 without the 1 -) at time ts, 0 outside the transit; bad on a Kepler failure.
+__device__ __forceinline__ double delta64(const PvHead<double>& H, const PvPb<double>& pbc,
+                                          const double* __restrict__ row, int ng, double ts, bool& bad) {
+    double tau = ts - H.T0;
+    tau = fma(-rint(tau * H.invP), H.P, tau);
+    const double dM = H.n * tau;
+    if (!abs_le64(dM, pbc.win_s)) return 0.0;
+    const Orbit64 o = orbit64(H, dM);
+    if (!o.ok) {
+        bad = true;
+        return __longlong_as_double(0x7ff8000000000000ll);
+    }
+    const double g = o.z * pbc.inv1pk;
+    if (!o.front || __double2hiint(g) >= 0x3ff00000) return 0.0;   // g >= 1
+    double d0, d1, sl;
+    int cell;
+    const double A = covered_area<double, false>(pbc.k, o.z, d0, d1);
+    return __dmul_rn(A, lerp_row<double>(row, ng, g, sl, cell));
+}
+
+// Constant output rows of one FP64 group (1 and NaN) in shared memory, sources of bulk stores, and the
+// output of a group's pvs outside their windows.
+struct ConstRows64 {
+    double *one, *nan_;
+    uint64_t pol;
+    // base: 2 n doubles, 16-byte aligned; a __syncthreads() follows before the first store
+    __device__ __forceinline__ void init(double* base, int n) {
+        one = base;
+        nan_ = base + n;
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            one[j] = 1.0;
+            nan_[j] = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        fence_proxy_async_smem();
+        pol = l2_evict_first_policy();
+    }
+    // out: the group's first time of the tile's first pv
+    template <int Q>
+    __device__ __forceinline__ void store(const Times64<Q>& T, int full, unsigned may, unsigned bad, int npv_t, int npb,
+                                          double* out, int npt, int bulk) const {
+        const int lane = threadIdx.x & 31;
+        const double nanv = __longlong_as_double(0x7ff8000000000000ll);
+        unsigned rest = (npv_t >= 32 ? 0xffffffffu : ((1u << npv_t) - 1u)) & ~may;
+        if (bulk && full) {
+            // one bulk store of the group's row per pv outside its windows (16-byte aligned: npt even, aligned flux)
+            if ((rest >> lane) & 1u) {
+                bulk_s2g(out + (size_t)lane * npt, ((bad >> lane) & 1u) ? nan_ : one, 32 * Q * sizeof(double), pol);
+                bulk_commit();
+            }
+            return;
+        }
+        #pragma unroll 1
+        while (rest) {
+            const int i = __ffs(rest) - 1;
+            rest &= rest - 1u;
+            const bool inval = (bad >> i) & 1u;
+            double* o = out + (size_t)i * npt;
+            if (full) {
+                #pragma unroll
+                for (int q = 0; q < Q; ++q) __stcs(o + 32 * q + lane, inval ? nanv : 1.0);
+            } else {
+                #pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (T.pb[q] >= 0) __stcs(o + Q * lane + q, inval || T.pb[q] >= npb ? nanv : 1.0);
+            }
+        }
+    }
+};
 
 }  // namespace rr

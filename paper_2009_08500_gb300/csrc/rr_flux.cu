@@ -425,26 +425,6 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
 // 10,007 times 403 -> 100 us (1.06 million FP64 instructions of warps, 0.67 of the pipe's
 // rate), 200 x 5,000 with 10 sub-exposures 4,677 -> 183, 1 x 2,000 25.3 -> 13.8.
 
-// One sample: A Ib (Eq. 5 without the 1 -) at time ts, 0 outside the transit; bad on a Kepler failure.
-__device__ __forceinline__ double delta64(const PvHead<double>& H, const PvPb<double>& pbc,
-                                          const double* __restrict__ row, int ng, double ts, bool& bad) {
-    double tau = ts - H.T0;
-    tau = fma(-rint(tau * H.invP), H.P, tau);
-    const double dM = H.n * tau;
-    if (!abs_le64(dM, pbc.win_s)) return 0.0;
-    const Orbit64 o = orbit64(H, dM);
-    if (!o.ok) {
-        bad = true;
-        return __longlong_as_double(0x7ff8000000000000ll);
-    }
-    const double g = o.z * pbc.inv1pk;
-    if (!o.front || __double2hiint(g) >= 0x3ff00000) return 0.0;   // g >= 1
-    double d0, d1, sl;
-    int cell;
-    const double A = covered_area<double, false>(pbc.k, o.z, d0, d1);
-    return A * lerp_row<double>(row, ng, g, sl, cell);
-}
-
 template <bool SS1, int Q>
 __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double* __restrict__ times,
                                                                  const int32_t* __restrict__ pb_index, int npt, int npv,
@@ -467,20 +447,13 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
     const int npv_t = min(pv_tile, npv - pv0);
     char* qbase = recs + (size_t)pv_tile * L.head_bytes;
     const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
-    // constant output rows of one group (1 and NaN), sources of the bulk stores
-    double* rows1 = reinterpret_cast<double*>(qbase + queue_bytes(pv_tile * groups_per_cta));
-    double* rowsnan = rows1 + kPts;
     const double nan_ = __longlong_as_double(0x7ff8000000000000ll);
     queue_init(queue, tc, pv_tile * groups_per_cta, gbeg);
-    for (int j = tid; j < kPts; j += kBlock64) {
-        rows1[j] = 1.0;
-        rowsnan[j] = nan_;
-    }
-    fence_proxy_async_smem();
+    ConstRows64 cr;
+    cr.init(reinterpret_cast<double*>(qbase + queue_bytes(pv_tile * groups_per_cta)), kPts);
     stage_pb64(pbp, ps);
     if (!stage_to_smem(recs, records + (size_t)pv0 * L.head_bytes, (uint32_t)npv_t * (uint32_t)L.head_bytes, bar, err))
         return;
-    const uint64_t l2_pol = l2_evict_first_policy();
 
     auto do_group = [&](int g) {
         Times64<Q> T;
@@ -491,31 +464,7 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
         float4 cl;
         const unsigned may = group_decide64(gs, recs, L.head_bytes, npv_t, bad, cl);
         if (may) queue_push(queue, tc, may, g, cl);
-        unsigned rest = (npv_t >= 32 ? 0xffffffffu : ((1u << npv_t) - 1u)) & ~may;
-        if (bulk && gs.full) {
-            // one bulk store of the group's row per pv outside its windows (16-byte aligned: npt even, aligned flux)
-            if ((rest >> lane) & 1u) {
-                bulk_s2g(flux + (size_t)(pv0 + lane) * npt + (size_t)g * kPts,
-                         ((bad >> lane) & 1u) ? rowsnan : rows1, kPts * sizeof(double), l2_pol);
-                bulk_commit();
-            }
-            return;
-        }
-        #pragma unroll 1
-        while (rest) {
-            const int i = __ffs(rest) - 1;
-            rest &= rest - 1u;
-            const bool inval = (bad >> i) & 1u;
-            double* out = flux + (size_t)(pv0 + i) * npt + (size_t)g * kPts;
-            if (gs.full) {
-                #pragma unroll
-                for (int q = 0; q < Q; ++q) __stcs(out + 32 * q + lane, inval ? nan_ : 1.0);
-            } else {
-                #pragma unroll
-                for (int q = 0; q < Q; ++q)
-                    if (T.pb[q] >= 0) __stcs(out + Q * lane + q, inval || T.pb[q] >= L.npb ? nan_ : 1.0);
-            }
-        }
+        cr.store(T, gs.full, may, bad, npv_t, L.npb, flux + (size_t)pv0 * npt + (size_t)g * kPts, npt, bulk);
     };
 
     auto do_item = [&](int it, int key) {

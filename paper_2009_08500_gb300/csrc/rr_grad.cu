@@ -46,12 +46,16 @@ template <typename R, bool DEP>
 __device__ __forceinline__ void grad_sample(const PvHead<R>& H, const PvPb<R>& pbc,
                                             const R* __restrict__ rowblk, const RecLayout& L, R z, R f1, R f3,
                                             int i, R al, R Px, R Py, R S, R V, R psi_tot, R gb, GradAcc<R>& acc,
-                                            R* dep, int kslot, int uslot) {
+                                            R* dep, int kslot, int uslot, R* depth = nullptr) {
     const R one = R(1);
     R dAdz, dAdk;
     const R A = covered_area_f13<R, true>(pbc.k, z, f1, f3, dAdz, dAdk);
     const R d = __ldg(rowblk + L.ng_pad + i);         // row[i+1] - row[i]
     const R Ib = __ldg(rowblk + i) + al * d;
+    if (depth) {   // the light curve's: the row interpolated as lerp_row does
+        const R l0 = __ldg(rowblk + i);
+        *depth = A * (l0 + al * (__ldg(rowblk + i + 1) - l0));
+    }
     const R dIdg = d * R(L.ng - 1);
     const R* rk = rowblk + 2 * L.ng_pad;
     const R rk0 = __ldg(rk + i);
@@ -543,12 +547,17 @@ __global__ void __launch_bounds__(kBlock, 3) rr_grad_mixed_kernel(
 // chunks of kChunk64 groups; rr_grad_finish_kernel then forms the chunks' sums in the same order).
 // Bound by the FP64 pipe.  Measured: 512 pvs x 10,007 times 529 -> 159 us, 64 x 3,000 579 -> 48, 200 x
 // 5,000 with 10 sub-exposures 6,582 -> 211.
-template <bool DEP, bool SS1>
+// FLUX: the light curves too (one sample per time), with the bits of rr_flux_fp64_kernel: its samples are
+// this kernel's, and evaluating them twice on the FP64 pipe was a third of the work of both.
+// Both together, two kernels beside each other / one: 512 x 10,007 224 -> 170 us, 128 x 10,007 98 -> 82, 200 x 5,000 97 -> 82,
+// 1 x 500 19.3 -> 19.6 (with one launch less).
+template <bool DEP, bool SS1, bool FLUX = false>
 __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     const double* __restrict__ times, const int32_t* __restrict__ pb_index, int npt, int npv,
     PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta, int pergroup, const char* __restrict__ records,
     const char* __restrict__ rowsg, const double* __restrict__ gflux, double* __restrict__ partials, int nacc,
-    int chromatic, int32_t* __restrict__ pv_status, int* err) {
+    int chromatic, int32_t* __restrict__ pv_status, double* __restrict__ flux, int bulk, int* err) {
+    static_assert(SS1 || !FLUX, "light curves with the gradient: one sample per time");
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
     TileCounters* tc = reinterpret_cast<TileCounters*>(smem + kOff64Tc);
@@ -561,6 +570,8 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     char* qbase = reinterpret_cast<char*>(depcols + (DEP ? (size_t)(nacc - 6) * kBlock64 : 0));
     qbase += (16 - ((uintptr_t)(qbase - (char*)smem) & 15)) & 15;
     const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
+    ConstRows64 cr{};
+    if (FLUX) cr.init(reinterpret_cast<double*>(qbase + queue_bytes(pv_tile * groups_per_cta)), kWarpPts);
     const int ngroups = (npt + kWarpPts - 1) / kWarpPts;
     const int gbeg = blockIdx.y * groups_per_cta;
     const int gend = min(ngroups, gbeg + groups_per_cta);
@@ -583,6 +594,7 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
         float4 cl;
         const unsigned may = group_decide64(gs, recs, L.head_bytes, npv_t, bad, cl);
         if (may) queue_push(queue, tc, may, g, cl);
+        if (FLUX) cr.store(T, gs.full, may, bad, npv_t, L.npb, flux + (size_t)pv0 * npt + (size_t)g * kWarpPts, npt, bulk);
     };
 
     auto do_item = [&](int it, int key) {
@@ -596,6 +608,7 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
         const double* rows = reinterpret_cast<const double*>(rowsg + (size_t)(pv0 + i) * L.rows_bytes);
         const double* gf = gflux + (size_t)(pv0 + i) * npt + (size_t)g * kWarpPts + 4 * lane;
         unsigned cand = candidates64(T, H, PB, L.npb, c);
+        const unsigned inside = cand;
         double gbq[4];
         #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -605,7 +618,39 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
                 if (gbq[q] == 0.0) cand &= ~(1u << q);
             }
         }
-        if (!__any_sync(0xffffffffu, cand != 0)) return;
+        bool bad = false;
+        // light curves with the gradient: the item's times from its samples' depths, or, where a cotangent
+        // is zero (its time is not among the gradient's samples), from a pass of their own
+        double* out = FLUX ? flux + (size_t)(pv0 + i) * npt + (size_t)g * kWarpPts + 4 * lane : nullptr;
+        auto store_item = [&](unsigned in, int first) {
+            #pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (T.pb[q] < 0) continue;
+                double f = T.pb[q] < L.npb ? 1.0 : __longlong_as_double(0x7ff8000000000000ll);
+                if ((in >> q) & 1u) f = 1.0 - wl->v[first++];
+                __stcs(out + q, f);
+            }
+        };
+        const bool alone = FLUX && __any_sync(0xffffffffu, cand != inside);
+        if (alone) {
+            const double zero[4] = {};
+            int nc, bq;
+            build_list64<SS1, 4>(wl, inside, T, zero, ps, nc, bq);
+            #pragma unroll 1
+            for (int j = lane; j < nc; j += 32) {
+                const int pb = wl->ps[j] & 31;
+                wl->v[j] = delta64(H, PB[pb], rows + (size_t)pb * L.rows_per_pb * L.ng_pad, L.ng, wl->t[j], bad);
+            }
+            __syncwarp();
+            store_item(inside, bq);
+            __syncwarp();
+            if (bad && pv_status) atomicOr(pv_status + pv0 + i, RR_PV_KEPLER);
+            bad = false;   // (the gradient's own samples decide below)
+        }
+        if (!__any_sync(0xffffffffu, cand != 0)) {
+            if (FLUX && !alone) store_item(0u, 0);
+            return;
+        }
         GradAcc<double> acc;
         #pragma unroll
         for (int j = 0; j < 6; ++j) acc.o[j] = 0.0;
@@ -614,7 +659,7 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
         for (int j = 0; j < 4; ++j) acc.u[j] = 0.0;
         if (DEP)
             for (int j = 6; j < nacc; ++j) dep[(j - 6) * kBlock64] = 0.0;
-        bool any = false, bad = false;
+        bool any = false;
         int nc, bq;
         const int ns = build_list64<SS1, 4>(wl, cand, T, gbq, ps, nc, bq);
         #pragma unroll 1
@@ -637,24 +682,32 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
                 ts = wl->t[j] + (at >= 0 ? ps->off[at + sub] : sub_offset64(ps->exptime[pb], ps->ss[pb], sub));
             }
             const PvPb<double> pbc = PB[pb];
+            const double gb = wl->v[j];
+            if (FLUX) wl->v[j] = 0.0;
             const double tau = ts - H.T0;
             const double m = rint(tau * H.invP);
             const double tr = fma(-m, H.P, tau);
             const double dM = H.n * tr;
             if (!abs_le64(dM, pbc.win_s)) continue;
             const Orbit64 o = orbit64(H, dM);
-            if (!o.ok) { bad = true; continue; }
+            if (!o.ok) {
+                bad = true;
+                if (FLUX) wl->v[j] = __longlong_as_double(0x7ff8000000000000ll);
+                continue;
+            }
             const double gz = o.z * pbc.inv1pk;
             if (!o.front || __double2hiint(gz) >= 0x3ff00000) continue;   // gz >= 1
             const double psi_tot = m + tr * H.invP;
-            const double xg = gz * (double)(L.ng - 1);
+            const double xg = __dmul_rn(gz, (double)(L.ng - 1));
             const int cell = min((int)xg, L.ng - 2);
             grad_sample<double, DEP>(H, pbc, rows + (size_t)pb * L.rows_per_pb * L.ng_pad, L, o.z, (1.0 + pbc.k) - o.z,
                                      o.z - (1.0 - pbc.k), cell, xg - (double)cell, o.Px, o.Py, o.S, o.V, psi_tot,
-                                     wl->v[j], acc, dep, 6 + (chromatic ? pb : 0), 6 + nkp + pb * L.nldc);
+                                     gb, acc, dep, 6 + (chromatic ? pb : 0), 6 + nkp + pb * L.nldc, FLUX ? &wl->v[j] : nullptr);
             any = true;
         }
         __syncwarp();
+        if (FLUX && !alone) store_item(cand, bq);
+        if (FLUX) __syncwarp();   // (the sums below reuse the list)
         if (bad) {
             acc.o[0] = __longlong_as_double(0x7ff8000000000000ll);
             any = true;
@@ -678,6 +731,7 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     else
         cta_partials_groups<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, blockIdx.y, gridDim.y,
                                     partials);
+    if (FLUX) bulk_wait_all();   // the bulk stores read shared memory that ends with the CTA
 }
 
 // Sum the partial sums of each pv over its chunks in chunk order (FP64),
@@ -777,11 +831,13 @@ __global__ void __launch_bounds__(kFinishThreads) rr_grad_finish_kernel(
     }
 }
 
-static size_t grad_smem(int pv_tile, const RecLayout& L, int nacc, bool dep, size_t rsize, int slots, bool ss1) {
+static size_t grad_smem(int pv_tile, const RecLayout& L, int nacc, bool dep, size_t rsize, int slots, bool ss1, bool flux) {
     size_t s = (rsize == 8 ? kOff64Recs : (ss1 ? kOffRecs32Packed : kOffRecs32)) + (size_t)pv_tile * L.head_bytes +
                (size_t)pv_tile * slots * nacc * rsize;
     if (dep) s += (size_t)(nacc - 6) * (rsize == 8 ? kBlock64 : kBlock) * rsize;
     s = ((s + 15) & ~(size_t)15) + queue_bytes(pv_tile * slots);
+    // constant output rows of the FP64 kernel with light curves
+    if (flux) s += 2 * kWarpPts * sizeof(double);
     // FP32 kernel: the summaries of the CTA's groups and the sine table
     if (rsize == 4) s += (size_t)slots * sizeof(GroupInfo) + (size_t)kSvTabLen * sizeof(float4);
     return s;
@@ -838,10 +894,19 @@ static bool grad_dep(const rr_ctx* c) {
     return c->nparam > 11 || (c->cfg.npb > 1 && (c->cfg.chromatic || c->nldc > 0)) || shared_weights(c);
 }
 
+bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt) {
+    if (c->cfg.precision != RR_PREC_FP64 || npv < 1 || npt < 1) return false;
+    for (int pb = 0; ss && pb < c->cfg.npb; ++pb)
+        if (ss[pb] != 1) return false;
+    const GradCut k = grad_cut(c, npv, npt);
+    return grad_smem(k.pv_tile, make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true), grad_nacc(c), grad_dep(c), 8, k.gpc,
+                     true, true) <= kMaxSmem;
+}
+
 cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
-                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s) {
+                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s, void* flux) {
     const bool f64 = c->cfg.precision == RR_PREC_FP64;
     RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true)
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
@@ -854,7 +919,7 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     if (!grad_ordered(c, pbp, npv, npt)) pts_ord = nullptr;
     bool ss1 = true;
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
-    const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1);
+    const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1, flux != nullptr);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
     const dim3 grid(npvt, (k.ngroups + gpc - 1) / gpc);
@@ -867,9 +932,13 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
         if (e != cudaSuccess) return e;                                                                       \
         KERNEL<<<grid, kBlock64, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile, gpc, k.pergroup,      \
                                           (const char*)records, rowsg, (const double*)grad_flux,              \
-                                          (double*)partials, nacc, c->cfg.chromatic, pv_status, c->d_err);    \
+                                          (double*)partials, nacc, c->cfg.chromatic, pv_status, (double*)flux, bulk, c->d_err);    \
     } while (0)
-        if (dep) {
+        const int bulk = flux && npt % 2 == 0 && ((uintptr_t)flux & 15u) == 0 && in_device_memory(flux);
+        if (flux) {
+            if (dep) RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<true, true, true>));
+            else RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<false, true, true>));
+        } else if (dep) {
             if (ss1) RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<true, true>));
             else RR_LAUNCH_GRAD64((rr_grad_fp64_kernel<true, false>));
         } else {

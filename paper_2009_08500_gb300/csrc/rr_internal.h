@@ -325,7 +325,10 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
 cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
-                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s);
+                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s,
+                        void* flux = nullptr);
+// whether the adjoint kernel also writes the light curves (launch_grad's flux): FP64 form, one sample per time
+bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt);
 // whether the forward kernel (the records' layout) and the adjoint launch their time chunks heaviest first:
 // passbands of different supersampling, several chunks, and a launch that is not cut below the chunk
 bool flux_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt, bool grad_layout);

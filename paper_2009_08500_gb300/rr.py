@@ -436,7 +436,7 @@ class Model:
                       pv_status: Optional[torch.Tensor] = None, stream=None):
         """(flux, grad_params) of a batch prepared by :meth:`prepare`, for a cotangent known in advance
         (rr_evaluate_both_prepared): the adjoint on a second stream of the context, beside the
-        forward kernel; bitwise :meth:`evaluate` and :meth:`evaluate_grad` with ``prepared``."""
+        forward kernel, or (FP64, one sample per time) one kernel for both; bitwise :meth:`evaluate` and :meth:`evaluate_grad` with ``prepared``."""
         npt, npv = self._inputs(times, params, pb_index)
         self._cotangent(grad_flux, npv, npt)
         ss, ex, ssp, exp_ = self._sampling(supersampling, exptime)
