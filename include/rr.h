@@ -166,9 +166,12 @@ rr_status rr_build_weights(rr_ctx* ctx, void* stream);
  * passband-major. */
 int32_t rr_nparam(const rr_ctx* ctx);
 
-/* Device workspace (bytes) that rr_evaluate (with_grad = 0) or
- * rr_evaluate_grad (with_grad = 1) needs for npv parameter vectors and npt
- * times.  0 on bad arguments. */
+/* Device workspace (bytes) for rr_evaluate (with_grad = 0) or
+ * rr_evaluate_grad (with_grad = 1) with npv parameter vectors and npt
+ * times.  A workspace of a batch with no fewer vectors and times serves too:
+ * where a small batch's own size is larger (with_grad = 1: partial sums of a
+ * finely cut launch), less makes that launch slower, with the same results.
+ * 0 on bad arguments. */
 size_t rr_workspace_bytes(const rr_ctx* ctx, int32_t npv, int32_t npt, int32_t with_grad);
 
 /* Evaluate light curves: flux[pv][t] for every parameter vector and time --
@@ -498,7 +501,8 @@ int64_t rr_launch_count(const rr_ctx* ctx);
 #define RR_KERNEL_FLUX 3
 #define RR_KERNEL_GRAD 4
 #define RR_KERNEL_GRAD_REDUCE 5
-#define RR_KERNEL_POINTS 6    /* several passbands; with one, the per-time preparation is part of PV_SETUP */
+#define RR_KERNEL_POINTS 6    /* the order of the time chunks: passbands of different supersampling, launches of several
+                               * whole chunks (the per-time preparation is part of PV_SETUP) */
 #define RR_KERNEL_DIRECT 7    /* the direct model's per-call weight projections */
 #define RR_KERNEL_KINDS 8
 
@@ -518,7 +522,7 @@ rr_status rr_profile_read(rr_ctx* ctx, int32_t kind, double* total_ms, int64_t* 
  *   RR_COUNT_SAMPLES   their exposure sub-samples: offset and window test
  *   RR_COUNT_ORBIT     of those, samples inside the window: the orbit
  *   RR_COUNT_CIRCULAR  of the orbits, circular ones (no Kepler solve)
- *   RR_COUNT_NEWTON    Newton iterations of the FP32 Kepler solves
+ *   RR_COUNT_NEWTON    iterations of the FP32 Kepler solves (forward: of third order)
  *   RR_COUNT_TRANSIT   samples in transit: covered area and profile lookup
  *                      (the adjoint: with every partial derivative)
  *   RR_COUNT_LENS      of those, samples on the stellar limb (ingress and

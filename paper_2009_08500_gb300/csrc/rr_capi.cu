@@ -1,6 +1,7 @@
 // Host implementation of the C ABI declared in include/rr.h.
 #include <cmath>
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <string>
@@ -162,7 +163,7 @@ rr_status check_eval(rr_ctx* c, const double* times, const int32_t* pb_index, in
     if (npt == 0 || npv == 0) return RR_OK;
     if (!times || !params || !out) return fail(c, RR_EINVAL, "times, params and the output must be non-null");
     if (c->cfg.npb > 1 && !pb_index) return fail(c, RR_EINVAL, "pb_index is required when npb > 1");
-    const size_t need = rr_workspace_bytes(c, npv, npt, grad ? 1 : 0);
+    const size_t need = ws_layout(c, npv, npt, grad).least;
     if (!ws || ws_bytes < need) {
         char b[160];
         std::snprintf(b, sizeof b, "workspace too small: %zu bytes given, %zu needed", ws ? ws_bytes : (size_t)0, need);
@@ -199,8 +200,8 @@ WsLayout ws_layout(const rr_ctx* c, int npv, int npt, bool grad) {
     if (c->cfg.precision == RR_PREC_MIXED && c->cfg.npb > 1)
         off += align256((size_t)time_chunks(npt, groups_per_cta(npt)) * sizeof(int));
     w.part = off;
-    if (grad) off += align256(partials_bytes(c, npv, npt));
-    w.total = off > 0 ? off : 256;
+    w.least = std::max<size_t>(off + (grad ? align256(partials_bytes(c, npv, npt, false)) : 0), 256);
+    w.total = std::max<size_t>(off + (grad ? align256(partials_bytes(c, npv, npt, true)) : 0), 256);
     return w;
 }
 }  // namespace rr
@@ -302,14 +303,15 @@ rr_status evaluate_grad_impl(rr_ctx* c, const double* times, const int32_t* pb_i
     const WsLayout W = ws_layout(c, npv, npt, true);
     char* wb = (char*)ws;
     void* partials = wb + W.part;
+    const size_t part_bytes = ws_bytes - W.part;
     if ((e = timed(c, RR_KERNEL_GRAD, s, [&] {
              return launch_grad(c, times, pb_index, wb + W.pts_dt, wb + W.pts_pb, wb + W.pts_grp,
                                 c->cfg.npb > 1 ? wb + W.pts_ord : nullptr, npt, npv, pbp, ws, grad_flux, partials,
-                                pv_status, s, flux);
+                                part_bytes, pv_status, s, flux);
          })) != cudaSuccess)
         return cuda_fail(c, e, "adjoint kernel");
     if ((e = timed(c, RR_KERNEL_GRAD_REDUCE, s, [&] {
-             return launch_grad_reduce(c, npt, params, npv, ws, partials, grad_params, s);
+             return launch_grad_reduce(c, npt, params, npv, ws, partials, part_bytes, grad_params, s);
          })) != cudaSuccess)
         return cuda_fail(c, e, "adjoint reduction kernel");
     return RR_OK;
@@ -562,7 +564,8 @@ rr_status rr_evaluate_both_prepared(rr_ctx* c, const double* times, const int32_
     if (!c) return fail(nullptr, RR_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
     // FP64 form, one sample per time: one kernel for both
-    if (flux && grad_with_flux(c, ss, npv, npt))
+    const size_t part = c->tables_built && npv > 0 && npt > 0 ? ws_layout(c, npv, npt, true).part : 0;
+    if (flux && grad_with_flux(c, ss, npv, npt, ws_bytes > part ? ws_bytes - part : 0))
         return evaluate_grad_impl(c, times, pb_index, npt, params, npv, ss, exptime, grad_flux, grad_params, pv_status,
                                   const_cast<void*>(ws), ws_bytes, true, stream, flux);
     cudaError_t e = cudaSetDevice(c->cfg.device);

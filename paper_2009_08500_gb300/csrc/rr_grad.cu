@@ -851,7 +851,8 @@ struct GradCut {
     bool pergroup;
 };
 
-static GradCut grad_cut(const rr_ctx* c, int npv, int npt) {
+// part_bytes: the workspace's room for partial sums; where the per-group sums do not fit, whole chunks per CTA.
+static GradCut grad_cut(const rr_ctx* c, int npv, int npt, size_t part_bytes = SIZE_MAX) {
     const bool f64 = c->cfg.precision == RR_PREC_FP64;
     const RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true)
                             : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
@@ -870,6 +871,11 @@ static GradCut grad_cut(const rr_ctx* c, int npv, int npt) {
     if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
     else split32(c, k.ngroups, npv, true, k.gpc, k.pv_tile);
     k.pergroup = k.gpc < k.chunk;
+    if (k.pergroup && (size_t)npv * k.ngroups * grad_nacc(c) * (f64 ? 8 : 4) > part_bytes) {
+        k.gpc = k.chunk;
+        k.pv_tile = tile(k.gpc);
+        k.pergroup = false;
+    }
     return k;
 }
 
@@ -879,10 +885,10 @@ bool grad_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt) {
     return k.gpc == k.chunk && k.nchunks > 1;
 }
 
-size_t partials_bytes(const rr_ctx* c, int npv, int npt) {
+size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool cut) {
     const size_t rsize = c->cfg.precision == RR_PREC_FP64 ? sizeof(double) : sizeof(float);
     const GradCut k = grad_cut(c, npv, npt);
-    return (size_t)npv * (size_t)(k.pergroup ? k.ngroups : k.nchunks) * (size_t)grad_nacc(c) * rsize;
+    return (size_t)npv * (size_t)(cut && k.pergroup ? k.ngroups : k.nchunks) * (size_t)grad_nacc(c) * rsize;
 }
 
 template <typename K>
@@ -894,11 +900,11 @@ static bool grad_dep(const rr_ctx* c) {
     return c->nparam > 11 || (c->cfg.npb > 1 && (c->cfg.chromatic || c->nldc > 0)) || shared_weights(c);
 }
 
-bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt) {
+bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt, size_t part_bytes) {
     if (c->cfg.precision != RR_PREC_FP64 || npv < 1 || npt < 1) return false;
     for (int pb = 0; ss && pb < c->cfg.npb; ++pb)
         if (ss[pb] != 1) return false;
-    const GradCut k = grad_cut(c, npv, npt);
+    const GradCut k = grad_cut(c, npv, npt, part_bytes);
     return grad_smem(k.pv_tile, make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true), grad_nacc(c), grad_dep(c), 8, k.gpc,
                      true, true) <= kMaxSmem;
 }
@@ -906,7 +912,8 @@ bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt) {
 cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
-                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s, void* flux) {
+                        const void* grad_flux, void* partials, size_t part_bytes, int32_t* pv_status, cudaStream_t s,
+                        void* flux) {
     const bool f64 = c->cfg.precision == RR_PREC_FP64;
     RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true)
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
@@ -914,7 +921,7 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     if (shared_weights(c)) L.kbar_slot = c->nparam;
     const bool dep = grad_dep(c);
     const size_t rsize = f64 ? 8 : 4;
-    const GradCut k = grad_cut(c, npv, npt);
+    const GradCut k = grad_cut(c, npv, npt, part_bytes);
     const int pv_tile = k.pv_tile, gpc = k.gpc;
     if (!grad_ordered(c, pbp, npv, npt)) pts_ord = nullptr;
     bool ss1 = true;
@@ -984,13 +991,13 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
 }
 
 cudaError_t launch_grad_reduce(rr_ctx* c, int npt, const double* params, int npv, const void* records,
-                               const void* partials, double* grad_params, cudaStream_t s) {
+                               const void* partials, size_t part_bytes, double* grad_params, cudaStream_t s) {
     const bool f64 = c->cfg.precision == RR_PREC_FP64;
     RecLayout L = f64 ? make_layout<double>(c->cfg.npb, c->cfg.ng, c->nldc, true)
                       : make_layout<float>(c->cfg.npb, c->cfg.ng, c->nldc, true);
     const int nacc = grad_nacc(c);
     const int shared = shared_weights(c) ? 1 : 0;
-    const GradCut k = grad_cut(c, npv, npt);
+    const GradCut k = grad_cut(c, npv, npt, part_bytes);
     const int ngr = k.pergroup ? k.ngroups : 0;
     const int nkp = c->cfg.chromatic ? c->cfg.npb : 1;
     const int kip = c->cfg.ld_model == RR_LD_QUADRATIC_TRI ? 1 : 0;

@@ -258,7 +258,9 @@ struct ReqLayout {
     size_t t, pb, p, f, st, ws, g, go, total, ws_bytes;
 };
 
-ReqLayout req_layout(const rr_ctx* c, int npv, int npt, bool grad) {
+// least: with the least workspace (ws_layout), which grows with npv and npt; a request whose scratch does not hold the
+// full one runs its launches uncut.
+ReqLayout req_layout(const rr_ctx* c, int npv, int npt, bool grad, bool least = false) {
     const size_t es = c->cfg.precision == RR_PREC_FP64 ? sizeof(double) : sizeof(float);
     ReqLayout L;
     L.t = 0;
@@ -267,7 +269,8 @@ ReqLayout req_layout(const rr_ctx* c, int npv, int npt, bool grad) {
     L.f = L.p + up256((size_t)npv * c->nparam * 8);
     L.st = L.f + up256((size_t)npv * npt * es);
     L.ws = L.st + up256((size_t)npv * 4);
-    L.ws_bytes = up256(rr_workspace_bytes(c, npv, npt, grad ? 1 : 0));
+    const WsLayout W = ws_layout(c, npv, npt, grad);
+    L.ws_bytes = up256(least ? W.least : W.total);
     L.g = L.ws + L.ws_bytes;
     L.go = L.g + (grad ? up256((size_t)npv * npt * es) : 0);
     L.total = L.go + (grad ? up256((size_t)npv * c->nparam * 8) : 0);
@@ -284,8 +287,9 @@ extern "C" size_t rr_request_bytes(const rr_ctx* c, int32_t npv, int32_t npt, in
 extern "C" int32_t rr_host_path(const rr_ctx* c) { return c ? c->host_path : 0; }
 
 namespace rr {
-size_t request_bytes_in_place(const rr_ctx* c, int npv, int npt, bool grad) {
-    return npv > 0 && npt > 0 ? req_layout(c, npv, npt, grad).ws_bytes : req_layout(c, npv, npt, grad).total;
+size_t request_bytes_in_place(const rr_ctx* c, int npv, int npt, bool grad, bool least) {
+    const ReqLayout L = req_layout(c, npv, npt, grad, least);
+    return npv > 0 && npt > 0 ? L.ws_bytes : L.total;
 }
 }  // namespace rr
 
@@ -305,11 +309,12 @@ extern "C" rr_status rr_enqueue_host(rr_ctx* c, const double* times, const int32
         c->err = "rr_enqueue_host: a required host array is null";
         return RR_EINVAL;
     }
-    const ReqLayout L = req_layout(c, npv, npt, grad);
+    ReqLayout L = req_layout(c, npv, npt, grad);
     cudaError_t e = cudaSetDevice(c->cfg.device);
     if (e != cudaSuccess) return pipe_fail(c, e, "rr_enqueue_host");
     const InPlace m = map_in_place(c, times, pb_index, npt, params, npv, grad_flux, flux, grad_params, pv_status);
     // in place, the scratch holds the workspace only
+    if (scratch_bytes < (m.ok ? L.ws_bytes : L.total)) L = req_layout(c, npv, npt, grad, true);
     if (!scratch || scratch_bytes < (m.ok ? L.ws_bytes : L.total) || ((uintptr_t)scratch & 255u)) {
         c->err = "rr_enqueue_host: scratch too small or not 256-byte aligned";
         return RR_EINVAL;

@@ -325,10 +325,10 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
 cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
-                        const void* grad_flux, void* partials, int32_t* pv_status, cudaStream_t s,
+                        const void* grad_flux, void* partials, size_t part_bytes, int32_t* pv_status, cudaStream_t s,
                         void* flux = nullptr);
 // whether the adjoint kernel also writes the light curves (launch_grad's flux): FP64 form, one sample per time
-bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt);
+bool grad_with_flux(const rr_ctx* c, const int32_t* ss, int npv, int npt, size_t part_bytes);
 // whether the forward kernel (the records' layout) and the adjoint launch their time chunks heaviest first:
 // passbands of different supersampling, several chunks, and a launch that is not cut below the chunk
 bool flux_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt, bool grad_layout);
@@ -350,7 +350,7 @@ inline int time_chunks(int npt, int gpc) { return ((npt + kWarpPts - 1) / kWarpP
 const void* mapped_host(const void* p, size_t bytes);
 // Device scratch of one request whose host buffers are all mapped page-locked memory (the
 // workspace alone; rr_request_bytes is the staged figure).
-size_t request_bytes_in_place(const rr_ctx* c, int npv, int npt, bool grad);
+size_t request_bytes_in_place(const rr_ctx* c, int npv, int npt, bool grad, bool least = false);
 // Device addresses of every caller buffer of one evaluation, when all of them are mapped
 // page-locked memory (ok; looked up for the current device); a batch with no times or no pvs
 // is staged.
@@ -381,13 +381,16 @@ inline bool in_device_memory(const void* p) {
     return a.type == cudaMemoryTypeDevice;
 }
 cudaError_t launch_grad_reduce(rr_ctx* c, int npt, const double* params, int npv, const void* records,
-                               const void* partials, double* grad_params, cudaStream_t s);
+                               const void* partials, size_t part_bytes, double* grad_params, cudaStream_t s);
 size_t records_bytes(const rr_ctx* c, int npv, bool grad);
-size_t partials_bytes(const rr_ctx* c, int npv, int npt);
+// cut: with the per-group sums of a launch cut below the chunks
+size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool cut);
 // workspace layout: [records | direct-model projections | per-point float-float times + passband,
 //                    per-group summaries (mixed form) | partial sums]
 struct WsLayout {
     size_t rec, dir, pts_dt, pts_pb, pts_grp, pts_ord, part, total;
+    size_t least;   // what a call needs: the partial sums of uncut launches (grows with npv and npt, so that a workspace
+                    // of a larger batch serves a smaller one; a cut launch with less than total runs uncut)
 };
 WsLayout ws_layout(const rr_ctx* c, int npv, int npt, bool grad);
 

@@ -324,6 +324,7 @@ extern "C" int64_t rr_server_submit_at(rr_server* s, rr_ctx* fit, const double* 
     r.grad = grad_params;
     r.status = pv_status;
     r.bytes = rr::request_bytes_in_place(fit, npv, npt, grad_flux != nullptr);
+    if (r.bytes > s->budget) r.bytes = rr::request_bytes_in_place(fit, npv, npt, grad_flux != nullptr, true);
     if (r.bytes > s->budget) return -RR_ENOMEM;
     r.t_arrival = release_ns > 0 ? release_ns : now_ns();
     int64_t id;
