@@ -51,7 +51,7 @@ CONFIG_TEXT = {
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch, from one ncu capture
 # of the same kernels (profiles/flux_mixed_c4_heterogeneous.md, flux_mixed_c3_population.md,
 # grad_mixed_c3_population.md); to be cleared whenever those kernels change
-TRAFFIC = {("c4", "flux"): 448_615_168, ("c3", "flux"): 273_952_512, ("c3", "grad"): 39_271_680}
+TRAFFIC = {("c4", "flux"): 457_581_824, ("c3", "flux"): 274_606_336, ("c3", "grad"): 39_287_296}
 
 
 # Algorithmic FP32 operations (add, multiply, fused multiply-add: one each) and MUFU operations
@@ -64,6 +64,7 @@ TRAFFIC = {("c4", "flux"): 448_615_168, ("c3", "flux"): 273_952_512, ("c3", "gra
 #   orbit      P_x, P_y, z^2, square root, g                                            11 + 1 MUFU
 #   kepler     start of the FP32 solve (series inversion)                              4
 #   newton     one Newton step (S, V series, f, f', quotient, rotation, stop test)       26 + 1 MUFU
+#   step3      forward: one third-order step (f'' and the second-order rotation more)    36 + 1 MUFU
 #   circ       S and V series of a circular orbit                                      13
 #   transit    forward: the g-lerp of the profile row and the product (a planet wholly
 #              on the disk has the constant area pi k^2)                               5
@@ -72,7 +73,7 @@ TRAFFIC = {("c4", "flux"): 448_615_168, ("c3", "flux"): 273_952_512, ("c3", "gra
 #   transit_adj  adjoint: the lerps, the area and orbit partials, 9 accumulations      98 + 2 MUFU
 #   lens_adj   adjoint on the limb: the lens and its z- and k-derivatives              40 + 4 MUFU
 #   refined    float-float z, contact factors and g cell (contact_z_ff)                340 + 3 MUFU
-FP32_OPS = {"phase": 15, "sample": 7, "orbit": 11, "kepler": 4, "newton": 26, "circ": 13, "transit": 5,
+FP32_OPS = {"phase": 15, "sample": 7, "orbit": 11, "kepler": 4, "newton": 26, "step3": 36, "circ": 13, "transit": 5,
             "lens": 39, "transit_adj": 98, "lens_adj": 40, "refined": 340}
 MUFU_OPS = {"orbit": 1, "newton": 1, "lens": 3, "transit_adj": 2, "lens_adj": 4, "refined": 3}
 FP32_LANES_PER_SM, MUFU_LANES_PER_SM = 128, 16
@@ -82,7 +83,8 @@ def alu_ops(kind, c):
     """(FP32 ops, MUFU ops) of one launch from its sample counts (rr_count_read)."""
     ecc = c["orbit"] - c["circular"]
     f = (FP32_OPS["phase"] * c["cand"] + FP32_OPS["sample"] * c["samples"] + FP32_OPS["orbit"] * c["orbit"] +
-         FP32_OPS["kepler"] * ecc + FP32_OPS["newton"] * c["newton"] + FP32_OPS["circ"] * c["circular"])
+         FP32_OPS["kepler"] * ecc + FP32_OPS["step3" if kind == "flux" else "newton"] * c["newton"] +
+         FP32_OPS["circ"] * c["circular"])
     m = MUFU_OPS["orbit"] * c["orbit"] + MUFU_OPS["newton"] * c["newton"]
     if kind == "flux":
         f += FP32_OPS["transit"] * c["transit"] + FP32_OPS["lens"] * c["lens"]

@@ -10,21 +10,22 @@
 // row segments of exactly 1 for the pvs outside their windows (bulk
 // asynchronous stores from a constant shared-memory row), and a work item
 // (pv, group) in a shared-memory queue for the others; the remaining warps
-// evaluate the items as they appear (candidate samples compacted per warp,
-// 32 at a time).  FP64 kernel: the same groups and queue with CTAs of two
-// warps, transit decisions in FP32, every sample in FP64.
+// evaluate the items as they appear (candidate samples compacted per warp).
+// FP64 kernel: the same groups and queue with CTAs of two warps, transit
+// decisions in FP32, every sample in FP64.
 //
 // Mixed precision (FP32 bulk):
 //  * per time, once per call (points_group): dt = t - t_g in FP64, kept as
 //    a float pair (dh, dl) -- t_g is the first time of the time's group;
 //  * per (CTA, pv), FP64: A = frac((t_ref - T0) / P) as a float pair at the
-//    CTA's first group, carried to each group in float-float;
+//    first group of the CTA's chunk, carried to each group in float-float;
 //  * per (pv, time): coarse phase psi = A + dh / P with one FMA, rounded
 //    with two additions (no FP64, no conversion per point).  If the
 //    whole exposure lies outside the pv's transit window the point is 1
 //    exactly and nothing else is computed.  Otherwise the phase is formed in
-//    float-float (error ~1e-9 of a cycle) and every sub-exposure goes
-//    through Kepler (FP32 Newton in the offset form, FP64 above e = 0.8),
+//    float-float (error ~1e-9 of a cycle) and every sub-exposure (two at a
+//    time) goes through Kepler (FP32 third-order steps in the offset form,
+//    FP64 above e = 0.8),
 //    the projected distance, the covered area and the profile row lookup.
 // FP64 form: the same structure with every step in FP64 and the phase
 // reduced per sub-exposure as tau = t_s - T0 - P rint((t_s - T0) / P).

@@ -548,10 +548,10 @@ __global__ void __launch_bounds__(kDirWarps * 32) rr_direct_table_kernel(
 // edge_area that no lane of a warp needs (the closed forms outside the lens, the
 // small-angle series, the compensated factors when c >= 2k) are skipped.  Bound by instruction issue (79% of the
 // slots, 31.6 of 32 lanes).  Measured against a thread per node, quadratic law, 200 +
-// 300 annuli, 200 nodes: 1,000 pvs 328 -> 156 us (with dT/dk 339 -> 170), 16 pvs
-// 117 -> 33; 2,048 pvs 552 -> 338 with dT/dk and shared weights; nonlinear law (five
-// bases: two per lane) 4,096 pvs 953 -> 679; CTAs of 128 threads against 256: 343 and
-// 353 (bands differ, smaller CTAs leave fewer warps waiting for their longest).
+// 300 annuli, 200 nodes: 1,000 pvs 328 -> 153 us (two or eight lanes per node 179 and
+// 198), 16 pvs 117 -> 33; 2,048 pvs 552 -> 319 with dT/dk and shared weights; nonlinear
+// law (five bases: two per lane) 4,096 pvs 953 -> 679; CTAs of 128 threads against 256: 343
+// and 353 (bands differ, smaller CTAs leave fewer warps waiting for their longest).
 constexpr int kDirLanes = 4;
 constexpr int kDirCta = 128;                             // threads per CTA
 constexpr int kDirNodes = kDirCta / kDirLanes;          // nodes per CTA
