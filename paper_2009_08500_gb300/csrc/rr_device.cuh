@@ -335,13 +335,35 @@ __device__ __forceinline__ float kepler_start_f32(float dM, const float4 ke, con
     const float y = dM * ke.w;
     return fmaf(fmaf(ks.z, y, ks.y), y * y, y);
 }
+// Far from the root the third-order step leaves the basin that Newton's keeps (orbits of a (1 - e) below about
+// 1.43, a planet that passes close by the star, with e > 0.4, whose windows are wide: 2% of samples over a (1 - e)
+// in [1, 1.45], and 0.03% with Newton's), so a sample that two steps leave unfinished starts again with
+// Newton's steps inside a bracket of the root: |x - dM| = e |sin E - sin E0| <= 2 e, and the function grows with x.
 __device__ __forceinline__ bool kepler_offset3_f32(float dM, const float4 ke, const float4 ks, float& x, float& S, float& V,
                                                    int& iters) {
     x = kepler_start_f32(dM, ke, ks);
+    float lo = 0.0f, hi = 0.0f;
     #pragma unroll 1
-    for (iters = 1; iters <= 24; ++iters) {
+    for (iters = 1; iters <= 42; ++iters) {
         half_angle_SV(x, S, V);
-        if (kepler_step3_f32(dM, ke, ks.w, x, S, V)) return true;
+        if (iters <= 2) {
+            if (kepler_step3_f32(dM, ke, ks.w, x, S, V)) return true;
+            const float w = fmaf(2.001f, ke.x, 1e-6f);
+            lo = dM - w;
+            hi = dM + w;
+            if (iters == 2) x = dM;
+            continue;
+        }
+        const float C = 1.0f - V;
+        const float f = fmaf(ke.z, V, fmaf(-ke.y, S, x - dM));
+        const float dx = __fdividef(f, fmaf(ke.z, S, fmaf(-ke.y, C, 1.0f))), xn = x - dx;
+        if (f > 0.0f) hi = x; else lo = x;
+        const bool inside = xn >= lo && xn <= hi;
+        x = inside ? xn : 0.5f * (lo + hi);
+        const float S_old = S;
+        S = fmaf(-dx, C, S);
+        V = fmaf(-dx, S_old, V);
+        if (inside && ks.w * dx * dx <= fmaf(1.5e-8f, fabsf(x), 1e-37f)) return true;
     }
     return false;
 }
