@@ -29,6 +29,8 @@
 //    the projected distance, the covered area and the profile row lookup.
 // FP64 form: the same structure with every step in FP64 and the phase
 // reduced per sub-exposure as tau = t_s - T0 - P rint((t_s - T0) / P).
+#include <algorithm>
+
 #include "rr_device.cuh"
 
 namespace rr {
@@ -432,7 +434,8 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
                                                                  PbParams pbp, RecLayout L, int pv_tile, int groups_per_cta,
                                                                  const char* __restrict__ records,
                                                                  const char* __restrict__ rowsg, double* __restrict__ flux,
-                                                                 int32_t* __restrict__ pv_status, int bulk, int* err) {
+                                                                 int32_t* __restrict__ pv_status, int bulk, int sum_shift,
+                                                                 float inv_ss, int* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
     TileCounters* tc = reinterpret_cast<TileCounters*>(smem + kOff64Tc);
@@ -495,61 +498,70 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
                 }
                 __syncwarp();
             } else {
-                // the item's flattened samples in 32 contiguous runs, one per lane, as in the FP32 kernel: sums of
-                // candidates inside a run are final, a run's head and tail are combined in lane order
-                const int run = (ns + 31) >> 5;
-                const int e_beg = min(lane * run, ns), e_end = min(e_beg + run, ns);
-                int jh = -1, jt = -1;
-                double ph = 0.0, pt = 0.0;
-                if (e_beg < e_end) {
-                    int lo = 0, hi = nc - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if ((wl->ps[mid] >> 5) <= e_beg) lo = mid; else hi = mid - 1;
-                    }
-                    int j = lo, pw = wl->ps[j], next = wl->ps[j + 1] >> 5, pb = pw & 31;
-                    int sub = e_beg - (pw >> 5);
-                    double t = wl->t[j], part = 0.0;
-                    jh = j;
+                // The item's flattened samples, kWarpPts at a time into the list, neighbouring ones in neighbouring
+                // lanes; then a time's samples are added in an order of their indices alone (whatever other times
+                // the group holds, and whatever its size): 2^sum_shift lanes per candidate, each adding every
+                // 2^sum_shift-th sample in order, and a fixed tree over them.  A finished sum takes its time's place in
+                // the list; the one candidate open at the end of a pass is carried.  Against a contiguous run of the
+                // item's samples per lane (whose sums depended on where the runs were cut), a call: 200 pvs x 5,000
+                // times with 10 sub-exposures 384 -> 299 us (neighbouring samples take the same branches), 8 x 500 with
+                // 1,000 1,762 -> 894, 1 x 20,000 with 30 195 -> 203 (the sums' chain).
+                const int R = 1 << sum_shift;
+                int lo = 0, jc = 0;      // the lane's last candidate; the first unfinished one
+                double carry = 0.0;      // of candidate jc: the sum of residue lane % R so far
+                #pragma unroll 1
+                for (int e0 = 0; e0 < ns; e0 += kWarpPts) {
+                    const int e1 = min(ns, e0 + kWarpPts);
                     #pragma unroll 1
-                    for (int e = e_beg; e < e_end; ++e) {
-                        if (e == next) {
-                            if (j == jh) ph = part; else wl->v[j] = part;
-                            ++j;
-                            pw = wl->ps[j];
-                            next = wl->ps[j + 1] >> 5;
-                            pb = pw & 31;
-                            t = wl->t[j];
-                            sub = 0;
-                            part = 0.0;
+                    for (int e = e0 + lane; e < e1; e += 32) {
+                        // the candidate holding sample e: by division where every passband has as many (exact: e below
+                        // 2^17 and at least half a sample from a multiple of the count), else by bisection
+                        if (inv_ss > 0.0f) {
+                            lo = (int)(((float)e + 0.5f) * inv_ss);
+                        } else {
+                            int hi = nc - 1;
+                            while (lo < hi) {
+                                const int mid = (lo + hi + 1) >> 1;
+                                if ((wl->ps[mid] >> 5) <= e) lo = mid; else hi = mid - 1;
+                            }
                         }
-                        const int at = ps->first[pb];
+                        const int pw = wl->ps[lo], pb = pw & 31, sub = e - (pw >> 5), at = ps->first[pb];
                         const double off = at >= 0 ? ps->off[at + sub] : sub_offset64(ps->exptime[pb], ps->ss[pb], sub);
-                        part += delta64(H, PB[pb], row_of(pb), L.ng, t + off, bad);
-                        ++sub;
+                        wl->v[e - e0] = delta64(H, PB[pb], row_of(pb), L.ng, wl->t[lo] + off, bad);
                     }
-                    if (j == jh) ph = part; else { jt = j; pt = part; }
+                    __syncwarp();
+                    const int j1 = __shfl_sync(0xffffffffu, lo, (e1 - 1 - e0) & 31);   // the candidate of sample e1 - 1
+                    const bool open = (wl->ps[j1 + 1] >> 5) > e1;
+                    const int last = (j1 - jc) << sum_shift;
+                    double next = 0.0;
+                    #pragma unroll 1
+                    for (int u0 = 0; u0 < last + R; u0 += 32) {
+                        const int u = u0 + lane, j = jc + (u >> sum_shift), r = u & (R - 1);
+                        double a = j == jc ? carry : 0.0;
+                        int end = 0;
+                        if (j <= j1) {
+                            end = wl->ps[j + 1] >> 5;
+                            int e = (wl->ps[j] >> 5) + r;
+                            if (e < e0) e += ((e0 - e + R - 1) >> sum_shift) << sum_shift;
+                            #pragma unroll 4
+                            for (; e < min(end, e1); e += R) a += wl->v[e - e0];
+                        }
+                        double sum = a;
+                        for (int o = 1; o < R; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                        if (j <= j1 && r == 0 && end <= e1) wl->t[j] = sum;
+                        if (open && last >= u0 && last < u0 + 32)
+                            next = __shfl_sync(0xffffffffu, a, last - u0 + (lane & (R - 1)));
+                    }
+                    carry = next;
+                    jc = open ? j1 : j1 + 1;
+                    __syncwarp();
                 }
-                const int tprev_j = __shfl_up_sync(0xffffffffu, jt, 1);
-                const double tprev_p = __shfl_up_sync(0xffffffffu, pt, 1);
-                if (lane > 0 && jh >= 0 && tprev_j == jh) ph = tprev_p + ph;
-                const int hnext_j = __shfl_down_sync(0xffffffffu, jh, 1);
-                if (jt >= 0 && (lane == 31 || hnext_j != jt)) wl->v[jt] = pt;
-                double v = ph;
-                #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const double y = __shfl_up_sync(0xffffffffu, v, o);
-                    const int ky = __shfl_up_sync(0xffffffffu, jh, o);
-                    if (lane >= o && ky == jh) v = y + v;
-                }
-                if (jh >= 0 && (lane == 31 || hnext_j != jh)) wl->v[jh] = v;
-                __syncwarp();
             }
             int j = bq;
             #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 if ((cand >> q) & 1u) {
-                    f[q] = SS1 ? 1.0 - wl->v[j] : 1.0 - wl->v[j] / ps->ss[T.pb[q]];
+                    f[q] = SS1 ? 1.0 - wl->v[j] : 1.0 - wl->t[j] / ps->ss[T.pb[q]];
                     ++j;
                 }
             }
@@ -731,8 +743,12 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const int bulk = npt % 2 == 0 && ((uintptr_t)flux & 15u) == 0 && in_device_memory(flux);
+        // lanes per candidate that add its samples: a function of the sub-exposures alone
+        const int ssmax = *std::max_element(pbp.ss, pbp.ss + pbp.npb);
+        const int sum_shift = ssmax < 4 ? 0 : (ssmax < 16 ? 1 : (ssmax < 64 ? 2 : 3));
         kern<<<grid, kBlock64, smem, s>>>(times, pb_index, npt, npv, pbp, L, pv_tile, gpc, (const char*)records, rowsg,
-                                          (double*)flux, pv_status, bulk, c->d_err);
+                                          (double*)flux, pv_status, bulk, sum_shift,
+                                          mixed_sampling(pbp) ? 0.0f : 1.0f / (float)pbp.ss[0], c->d_err);
     } else {
         auto kern = c->counting
                         ? (k.stage_rows ? (ss1 ? rr_flux_mixed_kernel<true, true, true>
