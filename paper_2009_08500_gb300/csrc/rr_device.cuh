@@ -1839,6 +1839,15 @@ constexpr int kBlock64 = 64;   // threads per CTA
 constexpr size_t kOff64Recs = kOff64Wl + (kBlock64 / 32) * kList64Bytes;
 static_assert(kOff64Wl % 16 == 0 && kOff64Recs % 16 == 0, "16-byte regions");
 
+// The CTA's tile of pvs and chunk of groups, tiles first (a grid of one dimension: see point_grid).
+struct Cta64 {
+    int tile, chunk;
+};
+__device__ __forceinline__ Cta64 cta64(int npv, int pv_tile) {
+    const int ntiles = (npv + pv_tile - 1) / pv_tile, chunk = (int)blockIdx.x / ntiles;
+    return {(int)blockIdx.x - chunk * ntiles, chunk};
+}
+
 // One sample: A Ib (Eq. 5 without the 1 -) at time ts, 0 outside the transit; bad on a Kepler failure.
 __device__ __forceinline__ double delta64(const PvHead<double>& H, const PvPb<double>& pbc,
                                           const double* __restrict__ row, int ng, double ts, bool& bad) {

@@ -445,9 +445,10 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
     List64* wl = reinterpret_cast<List64*>(smem + kOff64Wl + warp * kList64Bytes);
     constexpr int kPts = 32 * Q;   // times per group
     const int ngroups = (npt + kPts - 1) / kPts;
-    const int gbeg = blockIdx.y * groups_per_cta;
+    const Cta64 cta = cta64(npv, pv_tile);
+    const int gbeg = cta.chunk * groups_per_cta;
     const int gend = min(ngroups, gbeg + groups_per_cta);
-    const int pv0 = blockIdx.x * pv_tile;
+    const int pv0 = cta.tile * pv_tile;
     const int npv_t = min(pv_tile, npv - pv0);
     char* qbase = recs + (size_t)pv_tile * L.head_bytes;
     const ItemQueue queue = queue_at(qbase, pv_tile * groups_per_cta);
@@ -732,8 +733,8 @@ cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index,
     const size_t smem = flux_smem(pv_tile, k.per_pv, f64, gpc);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
-    const dim3 grid(npvt, (ngroups + gpc - 1) / gpc);
-    if (smem > kMaxSmem || grid.y > 65535u) return cudaErrorInvalidConfiguration;
+    const dim3 grid = point_grid(f64, npvt, (ngroups + gpc - 1) / gpc);
+    if (smem > kMaxSmem || grid.x == 0) return cudaErrorInvalidConfiguration;
     bool ss1 = true;
     for (int pb = 0; pb < pbp.npb; ++pb) ss1 = ss1 && pbp.ss[pb] == 1;
     cudaError_t e;

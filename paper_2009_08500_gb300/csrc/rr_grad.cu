@@ -573,9 +573,10 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     ConstRows64 cr{};
     if (FLUX) cr.init(reinterpret_cast<double*>(qbase + queue_bytes(pv_tile * groups_per_cta)), kWarpPts);
     const int ngroups = (npt + kWarpPts - 1) / kWarpPts;
-    const int gbeg = blockIdx.y * groups_per_cta;
+    const Cta64 cta = cta64(npv, pv_tile);
+    const int gbeg = cta.chunk * groups_per_cta;
     const int gend = min(ngroups, gbeg + groups_per_cta);
-    const int pv0 = blockIdx.x * pv_tile;
+    const int pv0 = cta.tile * pv_tile;
     const int npv_t = min(pv_tile, npv - pv0);
     queue_init(queue, tc, pv_tile * groups_per_cta, gbeg);
     stage_pb64(pbp, ps);
@@ -729,8 +730,8 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_grad_fp64_kernel(
     if (pergroup)
         cta_group_sums<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, gbeg, gend, ngroups, partials);
     else
-        cta_partials_groups<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, blockIdx.y, gridDim.y,
-                                    partials);
+        cta_partials_groups<double>(gacc, recs, L.head_bytes, npv_t, nacc, groups_per_cta, pv0, cta.chunk,
+                                    (ngroups + groups_per_cta - 1) / groups_per_cta, partials);
     if (FLUX) bulk_wait_all();   // the bulk stores read shared memory that ends with the CTA
 }
 
@@ -929,8 +930,8 @@ cudaError_t launch_grad(rr_ctx* c, const double* times, const int32_t* pb_index,
     const size_t smem = grad_smem(pv_tile, L, nacc, dep, rsize, gpc, ss1, flux != nullptr);
     const char* rowsg = (const char*)records + rows_offset(L, npv);
     const int npvt = (npv + pv_tile - 1) / pv_tile;
-    const dim3 grid(npvt, (k.ngroups + gpc - 1) / gpc);
-    if (smem > kMaxSmem || grid.y > 65535u) return cudaErrorInvalidConfiguration;
+    const dim3 grid = point_grid(f64, npvt, (k.ngroups + gpc - 1) / gpc);
+    if (smem > kMaxSmem || grid.x == 0) return cudaErrorInvalidConfiguration;
     cudaError_t e;
     if (f64) {
 #define RR_LAUNCH_GRAD64(KERNEL)                                                                              \

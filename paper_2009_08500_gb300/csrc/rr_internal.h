@@ -339,6 +339,13 @@ inline bool mixed_sampling(const PbParams& pbp) {
     return false;
 }
 cudaError_t launch_chunk_order(rr_ctx* c, int npt, void* ws_grp, void* ws_ord, cudaStream_t s);
+// The grid of a per-point launch: (pv tiles, chunks of groups), for the FP64 kernels, whose chunks stay short however
+// long the series is, in one dimension (65,535 chunks of 1,024 times would end at 67 million).  x = 0: too many.
+inline dim3 point_grid(bool f64, int tiles, int chunks) {
+    if (!f64) return chunks > 65535 ? dim3(0) : dim3(tiles, chunks);
+    const long long n = (long long)tiles * chunks;
+    return n > 0x7fffffffLL ? dim3(0) : dim3((unsigned)n);
+}
 // time chunks of the FP32 per-point kernels
 inline int time_chunks(int npt, int gpc) { return ((npt + kWarpPts - 1) / kWarpPts + gpc - 1) / gpc; }
 // Whether p is device memory.  A caller's buffer may also be page-locked host memory, which the
