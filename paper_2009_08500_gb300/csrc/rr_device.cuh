@@ -14,20 +14,23 @@ namespace rr {
 // dependent chain in a small one.  The functions below are written for both.
 //
 // Comparisons go through the bits (an FP64 comparison is an FP64 instruction too):
-// |x| <= y (false for a NaN x or y < 0), and the sign of a non-NaN x.
+// |x| <= y (false for a NaN x or y < 0; shifted, not masked: a mask of the sign becomes the
+// hardware's absolute value, which gives a NaN its sign back), and the sign of a non-NaN x.
 __device__ __forceinline__ bool abs_le64(double x, double y) {
-    return (__double_as_longlong(x) & 0x7fffffffffffffffll) <= __double_as_longlong(y);
+    const unsigned long long a = (unsigned long long)__double_as_longlong(x) << 1;
+    return a <= ((unsigned long long)__double_as_longlong(y) << 1) && __double2hiint(y) >= 0;
 }
 __device__ __forceinline__ bool neg64(double x) { return __double2hiint(x) < 0; }
 
-// Quotient of finite operands whose result and reciprocal are normal: the hardware's
-// approximate reciprocal (about 20 bits), one Newton-Raphson step, and the quotient
-// corrected by its exact remainder; within an ulp.
+// Reciprocal of d from the hardware's approximate one (about 20 bits) and one Newton-Raphson
+// step: within 2^-39 of its value.
 __device__ __forceinline__ double rcp64(double d) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     return fma(r, fma(-d, r, 1.0), r);
 }
+// Quotient of finite operands whose result and reciprocal are normal: the reciprocal's product
+// corrected by its exact remainder; within an ulp.
 __device__ __forceinline__ double div64(double n, double d) {
     const double r = rcp64(d), q = n * r;
     return fma(fma(-d, q, n), r, q);
