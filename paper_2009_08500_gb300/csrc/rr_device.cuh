@@ -1731,7 +1731,8 @@ __device__ __forceinline__ void group_state64(const Times64<Q>& T, int npb, cons
     bool whole = true;
     #pragma unroll
     for (int q = 0; q < Q; ++q) {
-        if (T.pb[q] >= 0 && isfinite(T.dh[q])) {
+        // (an offset beyond FP32's range widens the margins to every phase: group_decide64, candidates64)
+        if (T.pb[q] >= 0 && isfinite(T.t[q])) {
             lo = fminf(lo, T.dh[q]);
             hi = fmaxf(hi, T.dh[q]);
         }
@@ -1749,13 +1750,16 @@ __device__ __forceinline__ void group_state64(const Times64<Q>& T, int npb, cons
     if (lane < npv_t) {
         const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(recs + (size_t)lane * rec_bytes);
         if (H.status == 0) {
-            const double psi = (T.tref - H.T0) * H.invP;
-            gs.Ah = (float)(psi - rint(psi));
+            // reduced as the samples' own phases are, exactly: (tref - T0) / P rounded once loses the phase of a
+            // reference time many periods from T0
+            const double tau = T.tref - H.T0;
+            gs.Ah = (float)(fma(-rint(tau * H.invP), H.P, tau) * H.invP);
         }
     }
 }
 
-// group_decide for FP64 records (the same test; cl.x = the phase, cl.w = its rounding bound in cycles).
+// group_decide for FP64 records (the same test, true where it cannot be formed; cl.x = the phase, cl.w = its rounding
+// bound in cycles).
 __device__ __forceinline__ unsigned group_decide64(const GroupState& gs, const char* recs, int rec_bytes, int npv_t,
                                                    unsigned& bad, float4& cl) {
     const int lane = threadIdx.x & 31;
@@ -1768,7 +1772,7 @@ __device__ __forceinline__ unsigned group_decide64(const GroupState& gs, const c
         cl.w = 2.4e-7f * (gs.maxdt * Bh + 1.0f);
         if (!inval && gs.wlo <= gs.whi) {
             const float W = H.wmax_c + 2.0f * cl.w;
-            may = ceilf(fmaf(gs.wlo, Bh, cl.x) - W) <= fmaf(gs.whi, Bh, cl.x) + W;
+            may = !(ceilf(fmaf(gs.wlo, Bh, cl.x) - W) > fmaf(gs.whi, Bh, cl.x) + W);
         }
     }
     bad = __ballot_sync(0xffffffffu, inval);
@@ -1829,7 +1833,7 @@ __device__ __forceinline__ unsigned candidates64(const Times64<Q>& T, const PvHe
         if (pb < 0 || pb >= npb) continue;
         const float psi = fmaf(T.dh[q], Bh, c.x);
         const float d = psi - round_nearest(psi);
-        if (fabsf(d) <= PB[pb].win_pc + c.w) cand |= 1u << q;
+        if (!(fabsf(d) > PB[pb].win_pc + c.w)) cand |= 1u << q;   // (a phase that is not a number: the sample decides)
     }
     return cand;
 }
