@@ -198,7 +198,7 @@ WsLayout ws_layout(const rr_ctx* c, int npv, int npt, bool grad) {
     if (c->cfg.precision == RR_PREC_MIXED) off += align256((size_t)((npt + kWarpPts - 1) / kWarpPts) * sizeof(GroupInfo));
     w.pts_ord = off;
     if (c->cfg.precision == RR_PREC_MIXED && c->cfg.npb > 1)
-        off += align256((size_t)time_chunks(npt, groups_per_cta(npt)) * sizeof(int));
+        off += align256((size_t)most_time_chunks(npt, groups_per_cta(npt)) * sizeof(int));
     w.part = off;
     w.least = std::max<size_t>(off + (grad ? align256(partials_bytes(c, npv, npt, false)) : 0), 256);
     w.total = std::max<size_t>(off + (grad ? align256(partials_bytes(c, npv, npt, true)) : 0), 256);

@@ -886,10 +886,12 @@ bool grad_ordered(const rr_ctx* c, const PbParams& pbp, int npv, int npt) {
     return k.gpc == k.chunk && k.nchunks > 1;
 }
 
-size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool cut) {
-    const size_t rsize = c->cfg.precision == RR_PREC_FP64 ? sizeof(double) : sizeof(float);
+size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool full) {
+    const bool f64 = c->cfg.precision == RR_PREC_FP64;
     const GradCut k = grad_cut(c, npv, npt);
-    return (size_t)npv * (size_t)(cut && k.pergroup ? k.ngroups : k.nchunks) * (size_t)grad_nacc(c) * rsize;
+    int sums = k.nchunks;
+    if (full) sums = k.pergroup ? k.ngroups : (f64 ? k.nchunks : most_time_chunks(npt, k.chunk));
+    return (size_t)npv * (size_t)sums * (size_t)grad_nacc(c) * (f64 ? sizeof(double) : sizeof(float));
 }
 
 template <typename K>

@@ -258,8 +258,8 @@ struct ReqLayout {
     size_t t, pb, p, f, st, ws, g, go, total, ws_bytes;
 };
 
-// least: with the least workspace (ws_layout), which grows with npv and npt; a request whose scratch does not hold the
-// full one runs its launches uncut.
+// least: with the least workspace (ws_layout); a request whose scratch does not hold the full one, which
+// serves every smaller request too, runs its launches uncut.
 ReqLayout req_layout(const rr_ctx* c, int npv, int npt, bool grad, bool least = false) {
     const size_t es = c->cfg.precision == RR_PREC_FP64 ? sizeof(double) : sizeof(float);
     ReqLayout L;

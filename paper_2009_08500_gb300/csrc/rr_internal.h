@@ -18,6 +18,7 @@
 //   rr_grad_finish_kernel  partial sums -> grad_params (fixed order), chain rules
 #pragma once
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -348,6 +349,11 @@ inline dim3 point_grid(bool f64, int tiles, int chunks) {
 }
 // time chunks of the FP32 per-point kernels
 inline int time_chunks(int npt, int gpc) { return ((npt + kWarpPts - 1) / kWarpPts + gpc - 1) / gpc; }
+// ... and the most of any series of up to npt times: the number falls where groups_per_cta steps up (15 chunks
+// at 15,360 times, 8 at 15,361 and after each later step, at most 12 before the next) until its last step
+inline int most_time_chunks(int npt, int gpc) {
+    return std::max(std::min((npt + kPtTile - 1) / kPtTile, 15), time_chunks(npt, gpc));
+}
 // Whether p is device memory.  A caller's buffer may also be page-locked host memory, which the
 // kernels reach in place over the host link with plain loads and stores; the bulk asynchronous
 // copy engine (stores from shared memory, L2 prefetches) is used on device memory only.
@@ -390,14 +396,15 @@ inline bool in_device_memory(const void* p) {
 cudaError_t launch_grad_reduce(rr_ctx* c, int npt, const double* params, int npv, const void* records,
                                const void* partials, size_t part_bytes, double* grad_params, cudaStream_t s);
 size_t records_bytes(const rr_ctx* c, int npv, bool grad);
-// cut: with the per-group sums of a launch cut below the chunks
-size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool cut);
+// room for partial sums: what an uncut launch needs, or (full) what any launch of up to npt times writes, the
+// per-group sums of a launch cut below the chunks among them
+size_t partials_bytes(const rr_ctx* c, int npv, int npt, bool full);
 // workspace layout: [records | direct-model projections | per-point float-float times + passband,
 //                    per-group summaries (mixed form) | partial sums]
 struct WsLayout {
     size_t rec, dir, pts_dt, pts_pb, pts_grp, pts_ord, part, total;
-    size_t least;   // what a call needs: the partial sums of uncut launches (grows with npv and npt, so that a workspace
-                    // of a larger batch serves a smaller one; a cut launch with less than total runs uncut)
+    size_t least;   // what this call needs: the partial sums of uncut launches (a cut launch with less than total runs
+                    // uncut); total is at least the least of every smaller batch (fewer pvs or times)
 };
 WsLayout ws_layout(const rr_ctx* c, int npv, int npt, bool grad);
 
