@@ -710,7 +710,7 @@ static FluxCut flux_cut(const rr_ctx* c, const RecLayout& L, int npv, int npt, b
     k.q1 = f64 && (long long)npv * k.ngroups < 16LL * c->num_sms;
     if (k.q1) k.ngroups = (npt + 31) / 32;
     if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
-    else split32(c, k.ngroups, npv, false, k.gpc, k.pv_tile);
+    else if (!c->shared_gpu) split32(c, k.ngroups, npv, false, k.gpc, k.pv_tile);
     k.uncut = !f64 && k.gpc == groups_per_cta(npt) && k.ngroups > k.gpc;
     return k;
 }

@@ -263,6 +263,7 @@ struct rr_ctx {
     // fork and join events, created on first use
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    bool shared_gpu = false;   // the current call's kernels run beside others' (a server's): the forward launch is not cut
     // host-buffer pipeline (rr_evaluate_host): copy-in, compute and copy-out
     // streams, per-slot events, one grow-only device buffer
     struct HostPipe {

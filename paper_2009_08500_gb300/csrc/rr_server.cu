@@ -104,8 +104,12 @@ void CUDART_CB wake_worker(void* arg) {
 // same time is reported by whichever of them takes the word first).
 __global__ void take_error_kernel(int* dev_word, int* host_word) { *host_word = atomicExch(dev_word, 0); }
 
-// Enqueue one admitted request on its slot's stream (lock not held).
-void enqueue(rr_server* s, Request& r, Slot& sl) {
+// Enqueue one admitted request on its slot's stream (lock not held).  others: other requests are in flight or
+// waiting.  Their kernels fill the GPU, and a forward launch cut until a lone one fills it only adds CTAs, each with its
+// own set-up (12 slots of mixed requests in closed loop: 3.66e10 points/s with whole launches, 3.41e10 with cut ones; a
+// lone 16 x 2,000 call 90 and 70 us).  The adjoint stays cut: whole, 3.53e10.  Results are the same bits.
+void enqueue(rr_server* s, Request& r, Slot& sl, bool others) {
+    r.fit->shared_gpu = others;
     void* scratch = nullptr;
     const size_t bytes = r.bytes > 0 ? r.bytes : 256;
     cudaError_t e = cudaMallocFromPoolAsync(&scratch, bytes, s->pool, sl.stream);
@@ -125,6 +129,7 @@ void enqueue(rr_server* s, Request& r, Slot& sl) {
     } else {
         r.result = RR_ENOMEM;
     }
+    r.fit->shared_gpu = false;
     if ((e = cudaEventRecord(sl.done, sl.stream)) != cudaSuccess && r.result == RR_OK) r.result = RR_ECUDA;
     cudaLaunchHostFunc(sl.stream, wake_worker, s);
 }
@@ -138,17 +143,20 @@ void admit(rr_server* s, std::unique_lock<std::mutex>& lk) {
         Request& r = s->reqs[s->queue.front()];
         if (r.t_arrival > now_ns()) break;                // in order: not released yet
         if (s->used + r.bytes > s->budget) break;        // in order: wait for memory
-        int slot = -1;
-        for (size_t i = 0; i < s->slots.size(); ++i)
-            if (s->slots[i].req < 0) { slot = (int)i; break; }
+        int slot = -1, busy = 0;
+        for (size_t i = 0; i < s->slots.size(); ++i) {
+            if (s->slots[i].req >= 0) ++busy;
+            else if (slot < 0) slot = (int)i;
+        }
         if (slot < 0) break;
         s->queue.pop_front();
+        const bool others = busy > 0 || (!s->queue.empty() && s->reqs[s->queue.front()].t_arrival <= now_ns());
         Slot& sl = s->slots[slot];
         r.t_admit = now_ns();
         s->used += r.bytes;
         sl.req = r.id;
         lk.unlock();
-        enqueue(s, r, sl);
+        enqueue(s, r, sl, others);
         lk.lock();
     }
 }

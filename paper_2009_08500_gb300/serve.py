@@ -14,9 +14,10 @@ server keeps every fit's model context -- its LD profiles and (k, g) tables
 * records arrival / admission / launch / finish times, points and bytes of
   every request (p50 / p99 latency and points/s come from these).
 
-Results do not depend on what else is in flight: each request runs the same
-kernels with the same tiling as it would alone (the adjoint's summation
-order depends on the request's own number of times only).
+Results do not depend on what else is in flight: each request gives the bits
+that it would give alone, however its launches are cut (a time's samples are
+added in an order of their own, and the adjoint's summation order depends on
+the request's own number of times only).
 
 The scheduling logic is backend-agnostic (``Backend``); ``CudaBackend`` runs
 requests through the library, tests may plug in a host-only backend.
