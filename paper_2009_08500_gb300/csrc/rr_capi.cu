@@ -223,8 +223,7 @@ cudaError_t run_setup(rr_ctx* c, const double* times, const int32_t* pb_index, i
     if (e != cudaSuccess) return e;
     // the per-pv set-up and (mixed form) the per-time preparation in one launch (measured: the
     // preparation then costs nothing on the population workload; with 8 passbands the set-up
-    // grows by 1.5 us and the step saves 4 us against a launch of its own); with several
-    // passbands the chunk ordering follows
+    // grows by 1.5 us and the step saves 4 us against a launch of its own)
     const WsLayout W = ws_layout(c, npv, npt, grad);
     char* wb = (char*)ws;
     e = timed(c, RR_KERNEL_PV_SETUP, s, [&] {

@@ -166,12 +166,10 @@ __device__ __forceinline__ float d_atan2(float y, float x) { return atan2_upper(
 __device__ __forceinline__ double d_atan2(double y, double x) { return atan2_upper64(y, x); }
 __device__ __forceinline__ void d_sincos(float x, float* s, float* c) { sincosf(x, s, c); }
 __device__ __forceinline__ void d_sincos(double x, double* s, double* c) { sincos(x, s, c); }
-__device__ __forceinline__ float d_rint(float x) { return rintf(x); }
-__device__ __forceinline__ double d_rint(double x) { return rint(x); }
 // Reciprocal: the approximate instruction in FP32 (within about an ulp; the
 // adjoint's per-sample 1 / z and 1 / (1 - e cos E), far from zero and from
 // the FP32 range limits, where the rounding-exact form's special-case handling
-// costs issue slots), an exact IEEE division in FP64.
+// costs issue slots), within an ulp in FP64 (div64).
 __device__ __forceinline__ float d_rcp(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -789,16 +787,6 @@ __device__ __forceinline__ FF contact_z_ff(const PvOrbitFF& O, const float4* __r
     return ff_fast_two_sum(zf, r * (0.5f / zf));
 }
 
-__device__ __forceinline__ float warp_max(float v) {
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-template <typename T>
-__device__ __forceinline__ T sel4(const T (&v)[4], int q) {
-    return q == 0 ? v[0] : (q == 1 ? v[1] : (q == 2 ? v[2] : v[3]));
-}
-
 // Thread t of a CTA owns the 4 consecutive times pt0 + 4t .. pt0 + 4t + 3.
 __device__ __forceinline__ void load_points(const float2* __restrict__ pdt, const int32_t* __restrict__ ppb,
                                             int p0, int npt, float (&dh)[4], float (&dl)[4], int (&pbv)[4]) {
@@ -931,43 +919,14 @@ __device__ __forceinline__ int build_list(WarpList* wl, unsigned cand, const flo
     return ns;
 }
 
-// Candidate list when every passband has one sample per time: a candidate
-// is a sample, so the list is built from one ballot per time slot of the
-// lanes (no scans) and holds the raw offsets (dh, dl), the passband and the
-// per-time weight gbq; the precise phase is formed where a sample is
-// evaluated.  The list keeps time order (lane-major), so that a chunk of 32
+// Candidate list of the adjoint when every passband has one sample per time: a
+// candidate is a sample, so the list is built from one ballot per time slot of
+// the lanes (no scans), in time order (lane-major), so that a chunk of 32
 // samples is a contiguous stretch of the transit and takes the same branches.
-// bq[q] gets the list index of the lane's time q.  Returns the number of
-// candidates (warp-uniform).
-__device__ __forceinline__ int build_list_ss1(WarpList* wl, unsigned cand, const float (&dh)[4],
-                                              const float (&dl)[4], const int (&pbv)[4], const float (&gbq)[4],
-                                              int (&bq)[4]) {
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    int total = 0, before = 0;     // candidates of the whole warp / of the lanes below this one
-    #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const unsigned bal = __ballot_sync(0xffffffffu, (cand >> q) & 1u);
-        before += __popc(bal & below);
-        total += __popc(bal);
-    }
-    #pragma unroll
-    for (int q = 0; q < 4; ++q) bq[q] = before + __popc(cand & ((1u << q) - 1u));
-    #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if ((cand >> q) & 1u) {
-            wl->cand[bq[q]] = make_float4(dh[q], dl[q], 0.0f, gbq[q]);
-            wl->pb[bq[q]] = pbv[q];
-        }
-    }
-    __syncwarp();
-    return total;
-}
-
-// The same list for the adjoint, which needs neither the per-candidate sums
-// nor the sub-exposure offsets: one float4 per candidate (dh, dl, passband
-// index as int bits, gbq), 2 KB per warp instead of 3.6 KB, so that four CTAs
-// fit on an SM.
+// One float4 per candidate (the raw offsets dh and dl, the passband index as int
+// bits, the weight gbq; the precise phase is formed where a sample is evaluated):
+// 2 KB per warp, so that four CTAs fit on an SM.  Returns the number of candidates
+// (warp-uniform).
 __device__ __forceinline__ int build_list_ss1_packed(float4* wl, unsigned cand, const float (&dh)[4],
                                                      const float (&dl)[4], const int (&pbv)[4],
                                                      const float (&gbq)[4]) {
@@ -999,22 +958,6 @@ struct FluxList {
     float pacc[kWarpPts];
 };
 
-__device__ __forceinline__ int chunk_cand_ps(ChunkWalk& cw, const int* ps, int nc, int e0) {
-    const int lane = threadIdx.x & 31;
-    if (cw.jf + 1 < nc && (ps[cw.jf + 1] >> 5) <= e0) ++cw.jf;   // warp-uniform
-    const int jn = cw.jf + 1 + lane;
-    unsigned bit = 0u;
-    if (jn < nc) {
-        const int pos = (ps[jn] >> 5) - e0;
-        if (pos > 0 && pos < 32) bit = 1u << pos;
-    }
-    const unsigned starts = __reduce_or_sync(0xffffffffu, bit);
-    const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
-    const int j = cw.jf + __popc(starts & upto);
-    cw.jf = __shfl_sync(0xffffffffu, j, 31);
-    return j;
-}
-
 // build_list for the forward kernel (FluxList; returns the flattened sample count).
 __device__ __forceinline__ int build_list_flux(FluxList* fl, unsigned cand, const float (&dh)[4], const float (&dl)[4],
                                                const int (&pbv)[4], float Ah, float Al, float Bh, float Bl,
@@ -1044,7 +987,8 @@ __device__ __forceinline__ int build_list_flux(FluxList* fl, unsigned cand, cons
     return ns;
 }
 
-// build_list_ss1 for the forward kernel (FluxList: ps[j] = passband).
+// The same list (one ballot per time slot, in time order) for the forward kernel (FluxList: ps[j] = passband;
+// bq[q]: the list index of the lane's time q).
 __device__ __forceinline__ int build_list_ss1_flux(FluxList* fl, unsigned cand, const float (&dh)[4],
                                                    const float (&dl)[4], const int (&pbv)[4], int (&bq)[4]) {
     const int lane = threadIdx.x & 31;

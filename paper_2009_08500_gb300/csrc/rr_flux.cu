@@ -630,15 +630,17 @@ void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile) {
 }
 
 // The same for the FP32 kernels (gpc, pv_tile: the uncut launch's, kept from 3 CTAs per SM on): an
-// ensemble whose vectors transit together, or a few vectors, left most SMs without a CTA.  Pvs down to
-// 8 per CTA (an item per warp at least where every pv of the tile transits; 4 was slower) and parts of the
-// chunk (a multiple of 8 groups: a half, a quarter, an eighth, single groups), the forward kernel's groups
-// first, the adjoint's pvs first (its CTAs carry sums per (pv, group), and the finish kernel more partial
-// sums when the chunk is cut).  Measured, flux and adjoint: 16 pvs x 2,000 times 28.8 -> 11.8 and
+// ensemble whose vectors transit together, or a few vectors, left most SMs without a CTA.  Tiles of more
+// than 8 pvs are halved (an item per warp where every pv of 8 transits; tiles of 4 were slower; 9 to 15 pvs become
+// 5 to 8), and a CTA takes parts of the chunk (a multiple of 8 groups: a half, a quarter, an eighth, single groups),
+// the forward kernel's groups first, the adjoint's pvs first (its CTAs carry sums per (pv, group), and the finish
+// kernel more partial sums when the chunk is cut).  Measured, flux and adjoint: 16 pvs x 2,000 times 28.8 -> 11.8 and
 // 40.2 -> 13.9 us; 200 x 3,001 40.8 -> 12.8, 64.0 -> 19.4; 100 x 4,407 with 10 sub-exposures 69.1 ->
 // 13.5, 92.2 -> 17.5; 3 passbands, 256 x 9,001, adjoint 93.8 -> 35.2; prior populations 1,024 x 5,000
 // 24.9 -> 18.3, 33.1 -> 28.3.  With 6 CTAs per SM 1,024 x 5,000 takes 21.2 and 32.8, and tables staged
-// per CTA (256 pvs x 8 channels) 15.4 -> 18.3 from 4 on.
+// per CTA (256 pvs x 8 channels) 15.4 -> 18.3 from 4 on.  The price is the CTAs' own set-up where other streams
+// fill the GPU anyway (light curves on 8 to 12 streams at once, a call: 16 x 2,000 3.0 -> 1.4 us, 200 x 3,001 5.0 ->
+// 6.1, 500 x 5,000 8.3 -> 10.7, 64 x 20,000 3.7 -> 5.9): the server launches whole chunks (rr_server.cu).
 void split32(const rr_ctx* c, int ngroups, int npv, bool adjoint, int& gpc, int& pv_tile) {
     constexpr int min_tile = 8;
     const long long want = 3LL * c->num_sms;

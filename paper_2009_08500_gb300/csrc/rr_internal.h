@@ -9,7 +9,8 @@
 //                        pv's direct projections, or below k_small the profile at
 //                        the planet's centre); in the same launch (mixed form)
 //                        the per-time float-float offsets, passband and 128-time
-//                        group summaries; with several passbands then
+//                        group summaries; then, where passbands differ in
+//                        supersampling and a launch holds several whole chunks,
 //                        rr_chunk_order_kernel (time chunks heaviest first)
 //   rr_flux_mixed_kernel / rr_flux_fp64_kernel: records of a pv tile -> shared
 //                        memory (one bulk async copy), flux[pv][t] for the tile
@@ -94,14 +95,15 @@ template <typename R>
 struct alignas(16) PvPb {
     R k, inv1pk;      // radius ratio, 1 / (1 + k)
     R win_s;          // |dM| bound of a possible transit for one sample [rad]
-    R win_p;          // same, widened by the passband's exposure half-span [rad]
-    float win_pc;     // win_p in cycles (phase units of the FP32 point check)
+    R win_p;          // same, widened by the passband's exposure half-span [rad] (the fourth of the quadruple that
+                      // the kernels load; the point checks of both forms read win_pc)
+    float win_pc;     // win_p in cycles
     float cband;      // the mixed adjoint's contact band: kContactBand, or kContactBandGrazing
     float pad[2];
 };
 
 // Arguments of the per-time preparation carried by the set-up launch (its
-// first npoints CTAs; none when npt == 0).
+// last npoints CTAs, after the headers' and the rows'; none when npt == 0).
 struct PointsArgs {
     const double* times;
     const int32_t* pb_index;
@@ -310,7 +312,6 @@ cudaError_t launch_direct_tables(rr_ctx* c, const double* params, int npv, bool 
 size_t direct_bytes(const rr_ctx* c, int npv, bool grad);
 DirectTables direct_view(const rr_ctx* c, void* base, int npv, bool grad);
 cudaError_t launch_selftest(rr_ctx* c, int which, cudaStream_t s);
-// with several passbands also the order of the CTA time chunks, heaviest first (ws_ord)
 // records: the workspace (the direct model's projections follow the records).  With times
 // (mixed form, npt > 0) the same launch also writes the per-time inputs of the FP32 kernels
 // (float-float offsets, passband, 128-time group summaries) into pts_dt, pts_pb, pts_grp.
@@ -319,7 +320,7 @@ cudaError_t launch_pv_setup(rr_ctx* c, const double* params, int npv, const PbPa
                             const double* times = nullptr, const int32_t* pb_index = nullptr, int npt = 0,
                             void* pts_dt = nullptr, void* pts_pb = nullptr, void* pts_grp = nullptr);
 // grad_layout: the records were written in the adjoint's layout (rr_prepare)
-// pts_ord: the order of the time chunks (several passbands), or null (in index order)
+// pts_ord: room for the order of the time chunks (several passbands), or null; read where flux_ordered holds
 cudaError_t launch_flux(rr_ctx* c, const double* times, const int32_t* pb_index, const void* pts_dt,
                         const void* pts_pb, const void* pts_grp, const void* pts_ord, int npt, int npv,
                         const PbParams& pbp, const void* records,
@@ -382,7 +383,7 @@ InPlace map_in_place(const rr_ctx* c, const double* times, const int32_t* pb_ind
                      const double* params, int32_t npv, const void* grad_flux, void* flux, double* grad_params,
                      int32_t* pv_status);
 // One evaluation (with the adjoint when m.g is set) on mapped buffers, enqueued on s; ws is a
-// device workspace of ws_bytes >= rr_workspace_bytes.  overlap: the forward and adjoint kernels
+// device workspace of ws_bytes >= the least of ws_layout.  overlap: the forward and adjoint kernels
 // on s and the context's second stream (rr_evaluate_both_prepared).
 rr_status run_in_place(rr_ctx* c, const InPlace& m, int32_t npt, int32_t npv, const int32_t* ss,
                        const double* exptime, void* ws, size_t ws_bytes, cudaStream_t s, bool overlap);
