@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kBlock, 4) rr_flux_mixed_kernel(const double* 
 // CTAs of two warps: an item is a chain of ~6,000 cycles per 32 samples, and small CTAs keep
 // up to 16 items of an SM in flight without waiting for a CTA's longest.  Measured: 512 pvs x
 // 10,007 times 403 -> 100 us (1.06 million FP64 instructions of warps, 0.67 of the pipe's
-// rate), 200 x 5,000 with 10 sub-exposures 4,677 -> 183, 1 x 2,000 25.3 -> 13.8.
+// rate), 200 x 5,000 with 10 sub-exposures 4,686 -> 127, 1 x 2,000 24.3 -> 13.9.
 
 template <bool SS1, int Q>
 __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double* __restrict__ times,
@@ -504,9 +504,10 @@ __global__ void __launch_bounds__(kBlock64, 8) rr_flux_fp64_kernel(const double*
                 // the group holds, and whatever its size): 2^sum_shift lanes per candidate, each adding every
                 // 2^sum_shift-th sample in order, and a fixed tree over them.  A finished sum takes its time's place in
                 // the list; the one candidate open at the end of a pass is carried.  Against a contiguous run of the
-                // item's samples per lane (whose sums depended on where the runs were cut), a call: 200 pvs x 5,000
-                // times with 10 sub-exposures 384 -> 299 us (neighbouring samples take the same branches), 8 x 500 with
-                // 1,000 1,762 -> 894, 1 x 20,000 with 30 195 -> 203 (the sums' chain).
+                // item's samples per lane, whose sums depended on where the runs were cut (and whose lanes took different
+                // branches): 200 pvs x 5,000 times with 10 sub-exposures 176 -> 127 us, 64 x 3,000 103 -> 85, 1 x
+                // 20,000 with 30 52 -> 45, 8 x 500 with 1,000 3,930 -> 2,415; slower where one pv's transits are
+                // far apart and long (1 x 20,000 with 30 at random times, the call 195 -> 203: the sums' chain).
                 const int R = 1 << sum_shift;
                 int lo = 0, jc = 0;      // the lane's last candidate; the first unfinished one
                 double carry = 0.0;      // of candidate jc: the sum of residue lane % R so far
@@ -620,7 +621,7 @@ int pv_tile_for(int rec_bytes) {
 // Groups per CTA and pvs per CTA of the FP64 kernels.  An SM's FP64 work is what its CTAs hold, so
 // the launch is cut until there are 24 CTAs per SM, the groups first (at most 8: the adjoint's
 // chunk), then the pvs.  Measured at 1, 4, 16, 32 CTAs per SM: 512 pvs x 10,007 times 244, 135, 107, 103
-// us (adjoint 376, 215, 170, 163), 200 x 5,000 with 10 sub-exposures 487, 225, 196, 155.
+// us (adjoint 376, 215, 170, 163), 200 x 5,000 with 10 sub-exposures 389, 167, 128, 120.
 void split64(const rr_ctx* c, int ngroups, int npv, int& gpc, int& pv_tile) {
     const long long want = 24LL * c->num_sms;
     auto ctas = [&] { return (long long)((ngroups + gpc - 1) / gpc) * ((npv + pv_tile - 1) / pv_tile); };
@@ -708,7 +709,7 @@ static FluxCut flux_cut(const rr_ctx* c, const RecLayout& L, int npv, int npt, b
     k.ngroups = (npt + kWarpPts - 1) / kWarpPts;
     // FP64, few (pv, group) pairs: groups of 32 times, so that an item is one pass of its warp
     // (measured: 1 pv x 2,000 times 24.0 -> 13.8 us, 64 x 3,000 33.5 -> 29.4; 512 x 10,007 100 -> 96, but 200 x 5,000
-    // with 10 sub-exposures 180 -> 271: the candidates of 128 times fill a warp's passes better)
+    // with 10 sub-exposures 127 -> 197: the candidates of 128 times fill a warp's passes better)
     k.q1 = f64 && (long long)npv * k.ngroups < 16LL * c->num_sms;
     if (k.q1) k.ngroups = (npt + 31) / 32;
     if (f64) split64(c, k.ngroups, npv, k.gpc, k.pv_tile);
