@@ -36,3 +36,22 @@ def test_close_eccentric_orbits(ss, ex):
     wl.params = p[rows]
     ref = om.evaluate_workload(wl, om.build(wl.grid, wl.ld_model, wl.npb, wl.chromatic, wl.profiles, wl.n_general))
     assert (ref < 1).mean() > 0.05 and np.abs(f[rows] - ref).max() <= 1e-6
+
+
+def test_no_transit_is_lost_on_an_extreme_orbit():
+    """A planet whose orbit crosses the star (a = 1.137, e = 0.747, k = 0.807): a solve that runs off to infinity must not
+    pass for a planet out of transit.  FP32: 7e-7 in x, times a (1 + e) = 2 in z, times a slope of 0.8, some 1e-6; 5e-6."""
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2009_08500_gb300 import rr
+    wl = W.make_small("quadratic", npv=8, npt=3000, seed=3, direct=True)
+    p = wl.params
+    p[:, :7] = [0.87076078, 2.29136833, 1.13654818, 1.07053115, 0.74653325, 5.31471914, 0.80711502]
+    p[:, 5] += 0.02 * np.arange(8)
+    wl.times = np.sort(np.random.default_rng(4).uniform(0.0, 300.0, wl.npt))
+    m = rr.model_for(wl)
+    t, pb, dp = rr.to_device(wl)
+    f = m.evaluate(t, dp, pb).double().cpu().numpy()
+    m.sync_status()
+    ref = om.evaluate_workload(wl, om.build(wl.grid, wl.ld_model, wl.npb, wl.chromatic, wl.profiles, direct=True))
+    assert (ref < 1).mean() > 0.05 and np.abs(f - ref).max() <= 5e-6
