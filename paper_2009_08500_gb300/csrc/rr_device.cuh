@@ -1675,8 +1675,9 @@ __device__ __forceinline__ void group_state64(const Times64<Q>& T, int npb, cons
     bool whole = true;
     #pragma unroll
     for (int q = 0; q < Q; ++q) {
-        // (an offset beyond FP32's range widens the margins to every phase: group_decide64, candidates64)
-        if (T.pb[q] >= 0 && isfinite(T.t[q])) {
+        // (a NaN leaves both as they are; an infinite offset, of an infinite time or beyond FP32's range, widens the
+        // margins to every phase: group_decide64, candidates64)
+        if (T.pb[q] >= 0) {
             lo = fminf(lo, T.dh[q]);
             hi = fmaxf(hi, T.dh[q]);
         }
@@ -1694,10 +1695,11 @@ __device__ __forceinline__ void group_state64(const Times64<Q>& T, int npb, cons
     if (lane < npv_t) {
         const PvHead<double>& H = *reinterpret_cast<const PvHead<double>*>(recs + (size_t)lane * rec_bytes);
         if (H.status == 0) {
-            // reduced as the samples' own phases are, exactly: (tref - T0) / P rounded once loses the phase of a
-            // reference time many periods from T0
-            const double tau = T.tref - H.T0;
-            gs.Ah = (float)(fma(-rint(tau * H.invP), H.P, tau) * H.invP);
+            // within 1.5e-8 cycles up to 2^26 periods from T0; beyond, not a number: the samples decide, whose own phases
+            // are reduced exactly (so reduced here, for every pv, 200 pvs x 8,000 times took 61 us in place of 55)
+            const double psi = (T.tref - H.T0) * H.invP;
+            const float ph = (float)(psi - rint(psi));
+            gs.Ah = (__double2hiint(psi) & 0x7fffffff) < 0x41900000 ? ph : __int_as_float(0x7fc00000);
         }
     }
 }
