@@ -523,7 +523,7 @@ rr_status rr_profile_read(rr_ctx* ctx, int32_t kind, double* total_ms, int64_t* 
  *   RR_COUNT_ORBIT     of those, samples inside the window: the orbit
  *   RR_COUNT_CIRCULAR  of the orbits, circular ones (no Kepler solve)
  *   RR_COUNT_NEWTON    iterations of the FP32 Kepler solves (forward: of third order,
- *                      from the third on Newton's in a bracket)
+ *                      from the fourth on Newton's)
  *   RR_COUNT_TRANSIT   samples in transit: covered area and profile lookup
  *                      (the adjoint: with every partial derivative)
  *   RR_COUNT_LENS      of those, samples on the stellar limb (ingress and
