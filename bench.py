@@ -51,7 +51,7 @@ CONFIG_TEXT = {
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch, from one ncu capture
 # of the same kernels (profiles/flux_mixed_c4_heterogeneous.md, flux_mixed_c3_population.md,
 # grad_mixed_c3_population.md); to be cleared whenever those kernels change
-TRAFFIC = {("c4", "flux"): 457_779_968, ("c3", "flux"): 273_266_944, ("c3", "grad"): 39_287_296}
+TRAFFIC = {("c4", "flux"): 457_553_408, ("c3", "flux"): 273_716_480, ("c3", "grad"): 39_287_296}
 
 
 # Algorithmic FP32 operations (add, multiply, fused multiply-add: one each) and MUFU operations
